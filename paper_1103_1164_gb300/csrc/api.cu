@@ -104,6 +104,8 @@ dc::PlanView dc_plan::view() const
     for (int j = 0; j < 16; ++j) v.gw[j] = gw[j];
     v.merged_rt = merged ? 1 : 0;
     v.a_hi = (float)(coeffs.a_nt - 1);
+    v.inv_bx = 1.0f / bx;
+    v.inv_by = 1.0f / by;
     v.w_hi = (float)(coeffs.w_n - 1);
     v.item_rt = (coeffs.density_correction && lateral_mode != DC_LATERAL_ISO) ? 1 : 0;
     v.prec_rt = precision;
@@ -342,8 +344,8 @@ static dc_status upload_tables(dc_plan* p, const float* water, const float* dens
     for (int j = 0; j < c.w_n; ++j) {
         float a[8];
         for (int q = 0; q < 4; ++q) vs(q, j, &a[2 * q], &a[2 * q + 1]);
-        w[2 * j] = make_float4(a[0], a[1], a[2], a[3]);
-        w[2 * j + 1] = make_float4(a[4], a[5], a[6], a[7]);
+        w[j] = make_float4(a[0], a[1], a[2], a[3]);
+        w[c.w_n + j] = make_float4(a[4], a[5], a[6], a[7]);
     }
     DC_CUDA(cudaMemcpyAsync(p->d_water, w.data(), w.size() * sizeof(float4), cudaMemcpyHostToDevice, p->stream));
     DC_CUDA(cudaMemcpyAsync(p->d_dens, dens, sizeof(float) * 6 * (size_t)c.f_n, cudaMemcpyHostToDevice, p->stream));

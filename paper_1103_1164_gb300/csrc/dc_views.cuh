@@ -48,7 +48,9 @@ constexpr int kMaxBeams = 64;
 //   arow  [B][a_nt]    float2: (A_i, dA_i) at t_eq = j a_dt, where A_i is A
 //                      already interpolated at the beamlet's theta (the bilinear
 //                      lookup of A factors into theta then t_eq)
-//   water [w_n][2]     float4: (u1w, du1w, u2w, du2w), (w1w, dw1w, w2w, dw2w)
+//   water [2][w_n]     float4: (u1w, du1w, u2w, du2w), (w1w, dw1w, w2w, dw2w); two arrays, so that
+//                      a warp's lanes, at neighbouring samples, read 16 bytes apart (no bank
+//                      conflicts of the shared-memory copy)
 struct PlanView {
     int nx, ny, nz, n_beams, B, Kmax;
     float dx, dy, dz, ox, oy, oz;
@@ -83,6 +85,7 @@ struct PlanView {
     int item_rt;                  // lfac is in use
     int prec_rt;                  // direct-dose arithmetic (DC_PRECISION_*)
     float a_hi, w_hi;             // a_nt - 1, w_n - 1 as floats (clamps of the table coordinates)
+    float inv_bx, inv_by;         // 1 / beamlet size (window bounds)
     int32_t* chk;                 // status word of the DC_BOUNDS_CHECK build (first violated guard)
 };
 

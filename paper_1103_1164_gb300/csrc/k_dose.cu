@@ -85,6 +85,19 @@ __device__ __forceinline__ float rcp_approx(float x)
     return y;
 }
 
+// sqrt(x) to about one ulp, x >= 0.  The bounds of the beamlet windows take this
+// and the reciprocal beamlet sizes: they carry a margin of 1e-3 cm and the pair
+// test decides, while the IEEE square root and divisions, once per voxel and
+// beamlet row, took 3 % of the pair kernels' time (with the split water tables:
+// 2.44 -> 2.35 ms on the thorax plan of 516 M pairs, 11.5 -> 11.0 ms on a head
+// and neck plan of 2.47 G).
+__device__ __forceinline__ float sqrt_approx(float x)
+{
+    float y;
+    asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+
 // Table coordinates without a conversion instruction (conversions share the
 // quarter-rate pipe with the exponentials).  For 0 <= x < 2^22, adding
 // 1.5 * 2^23 with rounding toward -infinity leaves floor(x) in the low
@@ -220,7 +233,7 @@ __device__ __forceinline__ float pair_eval(const PlanView& P, const Lane& ln, co
         const float c2 = fmaf(fr, e1.y, e1.x);
         float fw;
         const uint32_t jw = DC_GUARD(P, grid_bits(fminf(t * P.inv_wdt, P.w_hi), fw) - kGridBits, P.w_n, 3);
-        const float4 w0 = sW[2 * jw], w1 = sW[2 * jw + 1];
+        const float4 w0 = sW[jw], w1 = sW[jw + P.w_n];
         u1w = fmaf(fw, w0.y, w0.x);
         u2w = fmaf(fw, w0.w, w0.z);
         O1 = fmaf(P.wscale, c1, fmaf(fw, w1.y, w1.x));
@@ -288,7 +301,7 @@ __device__ __forceinline__ void pair_grad(const PlanView& P, const float4 facv, 
     const float c2 = fmaf(fr, e1.y, e1.x);
     float fw;
     const int jw = (int)DC_GUARD(P, grid_bits(fminf(t * P.inv_wdt, P.w_hi), fw) - kGridBits, P.w_n, 3);
-    const float4 w0 = sW[2 * jw], w1 = sW[2 * jw + 1];
+    const float4 w0 = sW[jw], w1 = sW[jw + P.w_n];
     const float u1w = fmaf(fw, w0.y, w0.x), u2w = fmaf(fw, w0.w, w0.z);
     const float o1w = fmaf(fw, w1.y, w1.x), o2w = fmaf(fw, w1.w, w1.z);
     float fa;
@@ -489,8 +502,8 @@ __device__ __forceinline__ void process_unit(const DoseArgs& a, const int32_t vi
 
     int nlo = INT_MAX, nhi = INT_MIN;
     if (live) {
-        nlo = max(0, (int)ceilf((cc - rw + hfy) / P.by - 0.5f));
-        nhi = min(N - 1, (int)floorf((cc + rw + hfy) / P.by - 0.5f));
+        nlo = max(0, (int)ceilf(fmaf(cc - rw + hfy, P.inv_by, -0.5f)));
+        nhi = min(N - 1, (int)floorf(fmaf(cc + rw + hfy, P.inv_by, -0.5f)));
     }
     const int wnlo = __reduce_min_sync(0xffffffffu, nlo);
     const int wnhi = __reduce_max_sync(0xffffffffu, nhi);
@@ -499,9 +512,9 @@ __device__ __forceinline__ void process_unit(const DoseArgs& a, const int32_t vi
         const float h2 = rw * rw - dc_ * dc_;
         int mlo = INT_MAX, mhi = INT_MIN;
         if (live && h2 >= 0.f) {
-            const float hx = sqrtf(h2);
-            mlo = max(0, (int)ceilf((ca - hx + hfx) / P.bx - 0.5f));
-            mhi = min(M - 1, (int)floorf((ca + hx + hfx) / P.bx - 0.5f));
+            const float hx = sqrt_approx(h2);
+            mlo = max(0, (int)ceilf(fmaf(ca - hx + hfx, P.inv_bx, -0.5f)));
+            mhi = min(M - 1, (int)floorf(fmaf(ca + hx + hfx, P.inv_bx, -0.5f)));
         }
         const int wmlo = __reduce_min_sync(0xffffffffu, mlo);
         const int wmhi = __reduce_max_sync(0xffffffffu, mhi);
@@ -698,15 +711,18 @@ __device__ __forceinline__ void process_unit(const DoseArgs& a, const int32_t vi
 // Register budgets: 48 per thread for the single-fluence dose (5 CTAs per
 // SM), 64 for the pair count and the CSR fill (4 CTAs; the fill's extra state
 // would otherwise be recomputed in the hot loop), 80 for 16 fluence vectors,
-// 128 for 32 or 64 (their accumulators).
+// 128 for 32 or 64 (their accumulators).  A single-fluence dose whose units do
+// not fill the GPU takes 64 as well: its time is that of one unit's chain of
+// loads, and the two interleaved beamlets want the registers (4,320 voxels, 3
+// beams: 41 us with 48, 38 us with 64).
 template <int MODE, int NF>
 constexpr int min_ctas()
 {
     return MODE == kCount || MODE == kFill || MODE == kGrad ? 4 : (NF == 1 ? 5 : (NF == 16 ? 3 : 2));
 }
 
-template <int MODE, int NF, bool MERGED, int LAT, int PREC>
-__global__ void __launch_bounds__(kThreads, min_ctas<MODE, NF>()) k_pairs(const DoseArgs a)
+template <int MODE, int NF, bool MERGED, int LAT, int PREC, int MINB = min_ctas<MODE, NF>()>
+__global__ void __launch_bounds__(kThreads, MINB) k_pairs(const DoseArgs a)
 {
     extern __shared__ float4 smem[];
     __shared__ int64_t s_base[kMaxBeams + 1];
@@ -812,8 +828,8 @@ __device__ __forceinline__ void count_rows(const PlanView& P, const CountVoxel& 
     lo = INT_MAX;
     hi = INT_MIN;
     if (c.live) {
-        lo = max(0, (int)ceilf((c.cc - c.rw + hfy) / P.by - 0.5f));
-        hi = min(N - 1, (int)floorf((c.cc + c.rw + hfy) / P.by - 0.5f));
+        lo = max(0, (int)ceilf(fmaf(c.cc - c.rw + hfy, P.inv_by, -0.5f)));
+        hi = min(N - 1, (int)floorf(fmaf(c.cc + c.rw + hfy, P.inv_by, -0.5f)));
     }
 }
 
@@ -825,9 +841,9 @@ __device__ __forceinline__ void count_cols(const PlanView& P, const CountVoxel& 
     lo = INT_MAX;
     hi = INT_MIN;
     if (c.live && h2 >= 0.f) {
-        const float hx = sqrtf(h2);
-        lo = max(0, (int)ceilf((c.ca - hx + hfx) / P.bx - 0.5f));
-        hi = min(M - 1, (int)floorf((c.ca + hx + hfx) / P.bx - 0.5f));
+        const float hx = sqrt_approx(h2);
+        lo = max(0, (int)ceilf(fmaf(c.ca - hx + hfx, P.inv_bx, -0.5f)));
+        hi = min(M - 1, (int)floorf(fmaf(c.ca + hx + hfx, P.inv_bx, -0.5f)));
     }
 }
 
@@ -1091,8 +1107,8 @@ __device__ __forceinline__ void tile_unit(const DoseArgs& a, const PatchTiles& t
     const float rw = live ? (P.roi * sz_ * __ldg(&bm.inv_cos_max)) * 1.0005f + 1e-3f : 0.f;
     int nlo = INT_MAX, nhi = INT_MIN;
     if (live) {
-        nlo = max(0, (int)ceilf((cc - rw + hfy) / P.by - 0.5f));
-        nhi = min(N - 1, (int)floorf((cc + rw + hfy) / P.by - 0.5f));
+        nlo = max(0, (int)ceilf(fmaf(cc - rw + hfy, P.inv_by, -0.5f)));
+        nhi = min(N - 1, (int)floorf(fmaf(cc + rw + hfy, P.inv_by, -0.5f)));
     }
     const int wnlo = __reduce_min_sync(0xffffffffu, nlo);
     const int wnhi = __reduce_max_sync(0xffffffffu, nhi);
@@ -1112,9 +1128,9 @@ __device__ __forceinline__ void tile_unit(const DoseArgs& a, const PatchTiles& t
             const float dc_ = cc - (-hfy + (n + 0.5f) * P.by);
             const float h2 = rw * rw - dc_ * dc_;
             if (h2 < 0.f) continue;
-            const float hx = sqrtf(h2);
-            mlo = min(mlo, max(0, (int)ceilf((ca - hx + hfx) / P.bx - 0.5f)));
-            mhi = max(mhi, min(M - 1, (int)floorf((ca + hx + hfx) / P.bx - 0.5f)));
+            const float hx = sqrt_approx(h2);
+            mlo = min(mlo, max(0, (int)ceilf(fmaf(ca - hx + hfx, P.inv_bx, -0.5f))));
+            mhi = max(mhi, min(M - 1, (int)floorf(fmaf(ca + hx + hfx, P.inv_bx, -0.5f))));
         }
         const int wmlo = __reduce_min_sync(0xffffffffu, mlo);
         const int wmhi = __reduce_max_sync(0xffffffffu, mhi);
@@ -1491,12 +1507,15 @@ cudaError_t run_variant(const dc_plan* p, const DoseArgs& a)
 {
     const size_t sm = smem_bytes(p, MODE);
     auto kern = k_pairs<MODE, NF, MERGED, LAT, PREC>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    if (e != cudaSuccess) return e;
     int per_sm = 0, sms = 0;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kThreads, sm);
+    cudaError_t e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, p->device);
     if (e != cudaSuccess) return e;
-    e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, p->device);
+    // no more units than warps with 4 CTAs per SM
+    if (MODE == kDose && NF == 1 && (int64_t)p->n_beams * ((p->V + 31) / 32) <= (int64_t)sms * 4 * kWarps)
+        kern = k_pairs<MODE, NF, MERGED, LAT, PREC, MODE == kDose && NF == 1 ? 4 : min_ctas<MODE, NF>()>;
+    e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    if (e != cudaSuccess) return e;
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kThreads, sm);
     if (e != cudaSuccess) return e;
     e = cudaMemsetAsync(p->d_work + 1, 0, sizeof(int32_t), p->stream);
     if (e != cudaSuccess) return e;

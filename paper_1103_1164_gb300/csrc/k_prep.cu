@@ -320,7 +320,7 @@ __global__ void __launch_bounds__(256) k_merge_tables(const float4* __restrict__
         if (k >= __ldg(&bl[i].meta.x)) continue;
         const float4 a = __ldg(tab + 2 * e), b = __ldg(tab + 2 * e + 1);
         const int j = min(k, w_n - 1);
-        const float4 w0 = __ldg(water + 2 * j), w1 = __ldg(water + 2 * j + 1);
+        const float4 w0 = __ldg(water + j), w1 = __ldg(water + w_n + j);
         const float dw = k < w_n - 1 ? 1.f : 0.f;   // slope of the clamped water tables
         // values and slopes of the pairs (O1, O2) and (u1w, u2w) side by side,
         // for packed FP32 interpolation
