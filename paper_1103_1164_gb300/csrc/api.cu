@@ -122,7 +122,7 @@ static void free_plan(dc_plan* p)
                     p->d_bin, p->d_bounds, p->d_cellof, p->d_hist, p->d_nitems, p->d_bstart, p->d_bscan,
                     p->d_base, p->d_work,
                     p->d_items, p->d_part, p->d_bcount, p->d_sp_fp, p->d_sp_p, p->d_err,
-                    p->d_lfac, p->d_mlp_frag, p->d_mlp_bias, p->d_nfall, p->d_leaf, p->d_chk, p->d_grad};
+                    p->d_flupack, p->d_lfac, p->d_mlp_frag, p->d_mlp_bias, p->d_nfall, p->d_leaf, p->d_chk, p->d_grad};
     for (void* b : bufs)
         if (b) cudaFree(b);
     p->spmm_free();
@@ -683,6 +683,14 @@ dc_status dc_fspb_dose_batch(dc_plan* plan, const float* fluence, int32_t k, flo
         plan->sp_fp_cap = 0;
         DC_CUDA(dc::dev_malloc(&plan->d_sp_fp, (size_t)plan->B * 64 * sizeof(uint16_t)));
         plan->sp_fp_cap = (size_t)plan->B * 64;
+    }
+    const size_t need_pack = k > 1 && !tc ? (size_t)plan->B * dose_pass_width(k) : 0;
+    if (plan->flupack_cap < need_pack) {
+        if (plan->d_flupack) cudaFree(plan->d_flupack);
+        plan->d_flupack = nullptr;
+        plan->flupack_cap = 0;
+        DC_CUDA(dc::dev_malloc(&plan->d_flupack, need_pack * sizeof(float)));
+        plan->flupack_cap = need_pack;
     }
     // a single-fluence pass records the pair counts of the matrix pattern
     // while the pattern is unknown (every pair test is made there anyway)

@@ -128,18 +128,11 @@ cudaError_t enqueue(dc_batch* bt, bool density)
             if (e == cudaSuccess) e = launch_binning(p);
             if (e == cudaSuccess && p->coeffs.density_correction && p->lateral_mode != DC_LATERAL_ISO)
                 e = launch_lateral(p);
-            if (e == cudaSuccess) e = cudaMemsetAsync(p->d_part, 0, sizeof(float) * (size_t)p->n_beams * p->V, br);
             p->stream = own;
             if (e != cudaSuccess) return e;
             e = cudaEventRecord(bt->join[j], br);
             if (e != cudaSuccess) return e;
             e = cudaStreamWaitEvent(bt->cap, bt->join[j], 0);
-            if (e != cudaSuccess) return e;
-        }
-    } else if (bt->kvariant != kBatchPerPlan) {
-        for (int j = 0; j < bt->n; ++j) {
-            dc_plan* p = bt->plans[bt->order[j]];
-            e = cudaMemsetAsync(p->d_part, 0, sizeof(float) * (size_t)p->n_beams * p->V, bt->cap);
             if (e != cudaSuccess) return e;
         }
     }

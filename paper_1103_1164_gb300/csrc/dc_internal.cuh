@@ -75,8 +75,10 @@ struct dc_plan {
     int64_t* d_base = nullptr;       // [n_beams + 1] start of each beam's list (whole warps)
     int32_t* d_work = nullptr;       // [0] warp work units, [1] work counter
     int32_t* d_items = nullptr;      // [n_beams][V + 32]
-    float* d_part = nullptr;         // per-beam partial dose [n_beams][nf][V]
+    float* d_part = nullptr;         // per-beam partial dose [n_beams][V][vectors of a pass]
     size_t part_cap = 0;
+    float4* d_flupack = nullptr;     // the fluences of one multi-vector pass, [B][vectors]
+    size_t flupack_cap = 0;          // floats
     int32_t* d_bcount = nullptr;     // per-beam pair counts [n_beams][V]
     int persist_ctas[4] = {0, 0, 0, 0};
     // bumped whenever a buffer or a launch parameter that a captured batch

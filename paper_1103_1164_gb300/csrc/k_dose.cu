@@ -40,10 +40,6 @@ constexpr int kRingLd = kRing + 1;
 constexpr int row_max(int mode, int nf = 1) { return mode == 2 || nf > 32 ? 16 : 32; }
 
 enum Mode { kDose = 0, kCount = 1, kFill = 2, kGrad = 3 };
-// fluence vectors per pass of the dose kernel: 1, or 16, 32 or 64 staged
-// beside each beamlet record (as NF / 4 float4, whose order the staging
-// rotates by the lane's low two bits)
-constexpr bool valid_nf(int nf) { return nf == 1 || nf == 16 || nf == 32 || nf == 64; }
 
 // PREC 2, the tensor-core form of the multi-fluence dose (64 vectors): per
 // warp and chunk of 16 beamlets, Y[32 voxels][64] += D[32][16] F[16][64] as
@@ -436,7 +432,7 @@ __device__ __forceinline__ void flush_stage(const DoseArgs& a, const int2* st, i
 template <int MODE, int NF, bool MERGED, int LAT, int PREC = 0>
 __device__ __forceinline__ void process_unit(const DoseArgs& a, const int32_t vi, const int64_t e0, const int b,
                                              const float4* __restrict__ sW, int2* sst, float4* srow,
-                                             const int lane, float4* sflu = nullptr, uint32_t* stc = nullptr)
+                                             const int lane, uint32_t* stc = nullptr)
 {
     // the tensor-core form of 64 fluence vectors; its pair values in FP32
     // exponentials like the plain form
@@ -535,20 +531,6 @@ __device__ __forceinline__ void process_unit(const DoseArgs& a, const int32_t vi
             // theta weight (which only the table set-up uses)
             if (MODE != kCount && NF == 1) q2.w = __ldg(a.fluence + ib);
             srow[3 * lane + 2] = q2;
-            if (MODE == kDose && NF > 1 && !TC) {
-                // the beamlet's NF fluences beside its record (zero past a.nf),
-                // as NF / 4 float4 whose order is rotated by the lane (fewer
-                // bank conflicts among the lanes' stores)
-                float4* f4 = sflu + (NF / 4) * lane;
-#pragma unroll
-                for (int j = 0; j < NF / 4; ++j) {
-                    float f[4];
-#pragma unroll
-                    for (int h = 0; h < 4; ++h)
-                        f[h] = 4 * j + h < a.nf ? __ldg(a.fluence + ((4 * j + h) * (uint32_t)a.ldf + ib)) : 0.f;
-                    f4[j ^ (lane & 3)] = make_float4(f[0], f[1], f[2], f[3]);
-                }
-            }
         }
         if (TC) {
             // the chunk's 64 BF16 fluences of beamlets m0 + 2j and m0 + 2j + 1
@@ -604,22 +586,10 @@ __device__ __forceinline__ void process_unit(const DoseArgs& a, const int32_t vi
                 continue;
             }
             if (MODE == kDose) {
-                if (NF == 1) cnt += pt.in ? 1 : 0;
+                cnt += pt.in ? 1 : 0;
                 if (pt.in) {
                     const float D = pair_eval<MERGED, LAT, EP>(P, ln, i, sad, sW, pt);
-                    if (NF == 1) {
-                        acc[0] = fmaf(rq[2].w, D, acc[0]);
-                    } else {
-                        const float4* f4 = sflu + (NF / 4) * (m - m0);
-#pragma unroll
-                        for (int q4 = 0; q4 < NF / 4; ++q4) {
-                            const float4 f = f4[q4 ^ ((m - m0) & 3)];
-                            acc[4 * q4] = fmaf(f.x, D, acc[4 * q4]);
-                            acc[4 * q4 + 1] = fmaf(f.y, D, acc[4 * q4 + 1]);
-                            acc[4 * q4 + 2] = fmaf(f.z, D, acc[4 * q4 + 2]);
-                            acc[4 * q4 + 3] = fmaf(f.w, D, acc[4 * q4 + 3]);
-                        }
-                    }
+                    acc[0] = fmaf(rq[2].w, D, acc[0]);
                 }
             } else {
                 if (pt.in) {
@@ -684,21 +654,17 @@ __device__ __forceinline__ void process_unit(const DoseArgs& a, const int32_t vi
                 const int vr = __shfl_sync(0xffffffffu, vi, 16 * t + 8 * h + g);
 #pragma unroll
                 for (int u = 0; u < 8; ++u)
-#pragma unroll
-                    for (int e = 0; e < 2; ++e) {
-                        const int n = 8 * u + 2 * t4 + e;
-                        if (vr >= 0 && n < a.nf) a.part[((size_t)b * NF + n) * V + vr] = acc[(t * 8 + u) * 4 + 2 * h + e];
-                    }
+                    if (vr >= 0)
+                        *reinterpret_cast<float2*>(a.part + ((size_t)b * V + vr) * NF + 8 * u + 2 * t4) =
+                            make_float2(acc[(t * 8 + u) * 4 + 2 * h], acc[(t * 8 + u) * 4 + 2 * h + 1]);
             }
     } else if (MODE == kFill) {
         flush_stage(a, sst, lane, cnt, pos, pend, mis, true);
         if (NF == 1 && ln.valid) a.part[(size_t)b * V + v] = acc[0];
     } else if (ln.valid) {
         if (MODE == kDose) {
-#pragma unroll
-            for (int q = 0; q < NF; ++q)
-                if (q < a.nf) a.part[((size_t)b * NF + q) * V + v] = acc[q];
-            if (NF == 1 && a.count_out) a.count_out[(size_t)b * V + v] = cnt;
+            a.part[(size_t)b * V + v] = acc[0];
+            if (a.count_out) a.count_out[(size_t)b * V + v] = cnt;
         } else {
             a.bcount[(size_t)b * V + v] = cnt;
         }
@@ -710,15 +676,15 @@ __device__ __forceinline__ void process_unit(const DoseArgs& a, const int32_t vi
 // Persistent CTAs take units from a global counter.
 // Register budgets: 48 per thread for the single-fluence dose (5 CTAs per
 // SM), 64 for the pair count and the CSR fill (4 CTAs; the fill's extra state
-// would otherwise be recomputed in the hot loop), 80 for 16 fluence vectors,
-// 128 for 32 or 64 (their accumulators).  A single-fluence dose whose units do
+// would otherwise be recomputed in the hot loop), 128 for the tensor-core form of
+// 64 vectors (their accumulators).  A single-fluence dose whose units do
 // not fill the GPU takes 64 as well: its time is that of one unit's chain of
 // loads, and the two interleaved beamlets want the registers (4,320 voxels, 3
 // beams: 41 us with 48, 38 us with 64).
 template <int MODE, int NF>
 constexpr int min_ctas()
 {
-    return MODE == kCount || MODE == kFill || MODE == kGrad ? 4 : (NF == 1 ? 5 : (NF == 16 ? 3 : 2));
+    return MODE == kCount || MODE == kFill || MODE == kGrad ? 4 : (NF == 1 ? 5 : 2);
 }
 
 template <int MODE, int NF, bool MERGED, int LAT, int PREC, int MINB = min_ctas<MODE, NF>()>
@@ -739,12 +705,10 @@ __global__ void __launch_bounds__(kThreads, MINB) k_pairs(const DoseArgs a)
         sst = reinterpret_cast<int2*>(sgrad);
         for (int q = threadIdx.x; q < ngrad; q += blockDim.x) sgrad[q] = 0.f;
     }
-    static_assert(valid_nf(NF) || MODE != kDose, "16, 32 or 64 fluence vectors per pass");
+    static_assert(MODE != kDose || NF == (PREC == 2 ? 64 : 1), "one vector, or 64 in the tensor-core form");
     constexpr bool TC = MODE == kDose && PREC == 2;
     __shared__ float4 s_row[kWarps][3 * row_max(MODE, NF)];
-    // several fluence vectors: each staged beamlet's fluences (NF per record),
-    // or the tensor-core form's operand tiles
-    __shared__ float4 s_flu[NF > 1 && !TC ? kWarps : 1][NF > 1 && !TC ? row_max(MODE, NF) * NF / 4 : 1];
+    // the tensor-core form's operand tiles
     __shared__ __align__(16) uint32_t s_tc[TC ? kWarps : 1][TC ? kTcWords : 4];
     if (TC) {
         // columns past a partial chunk keep earlier (finite) pair values, which
@@ -768,7 +732,6 @@ __global__ void __launch_bounds__(kThreads, MINB) k_pairs(const DoseArgs a)
         while (b + 1 < P.n_beams && s_base[b + 1] <= e0) ++b;
         const int32_t vi = __ldg(a.items + e0 + lane);
         process_unit<MODE, NF, MERGED, LAT, PREC>(a, vi, e0, b, sW, sst, s_row[warp], lane,
-                                                  NF > 1 && !TC ? s_flu[NF > 1 && !TC ? warp : 0] : nullptr,
                                                   TC ? s_tc[TC ? warp : 0] : nullptr);
     }
     if (MODE == kGrad) {
@@ -1040,6 +1003,255 @@ __global__ void __launch_bounds__(kThreads, NV <= 2 ? 4 : (NV == 3 ? 3 : 2)) k_c
                 count_units<1>(a, ek, bk, s_row[warp], s_win[warp], lane);
             }
         }
+    }
+}
+
+// ---------------------------------------------------------------------------
+// Several fluence vectors in one FP32 pass.  Per unit of 32 voxels and 16
+// beamlets, the pair values D[16][32] are evaluated a voxel per lane into shared
+// memory (zero outside the pairs), and Y[32][NF] += D F is a register-tiled
+// product, 8 voxels x 2 or 4 vectors per lane, so a beamlet costs a lane 3
+// shared-memory vector loads for its 16 or 32 multiply-adds.  64 vectors take
+// two warps per unit, each evaluating every other beamlet and holding half of
+// the vectors.  Each sum runs over the beamlets in order, as the single-vector
+// pass's.  The fluences come packed as [B][NF] (zero past nf), the partial doses
+// go out as [n_beams][V][NF], whole lines per voxel.  Bound by issue slots and,
+// with the 24 or 32 warps per SM that the accumulators leave, by the latency of
+// the table loads: a call of 64 vectors on the thorax plan (516 M pairs) takes
+// 6.7 ms with one warp per unit, which leaves 16 warps, 6.3 ms with two, and took
+// 9.45 ms with a vector load per four multiply-adds.  32 vectors: 6.4 -> 4.4 ms,
+// 11 vectors: 4.0 -> 3.5 ms.
+constexpr int kMultiRows = 16;
+
+template <int NF>
+constexpr int multi_ctas()
+{
+    return NF == 16 ? 4 : 3;
+}
+
+// All threads of a unit's warps (pair `unit` of the CTA's warps, or one warp).
+template <int WPU>
+__device__ __forceinline__ void unit_sync(int unit)
+{
+    if (WPU == 1) __syncwarp();
+    else asm volatile("bar.sync %0, 64;" ::"r"(unit + 1) : "memory");
+}
+
+template <int NF, bool MERGED, int LAT>
+__global__ void __launch_bounds__(kThreads, multi_ctas<NF>()) k_dose_multi(const DoseArgs a)
+{
+    constexpr int WPU = NF == 64 ? 2 : 1;    // warps per unit
+    constexpr int NW = NF / WPU;             // vectors per warp
+    constexpr int VP = NW / 8;               // vectors per lane: 2 or 4
+    constexpr int kUnits = kWarps / WPU;     // units per CTA
+    extern __shared__ float4 smem[];
+    __shared__ int64_t s_base[kMaxBeams + 1];
+    __shared__ float4 s_row[kUnits][3 * kMultiRows];
+    __shared__ float4 s_d[kUnits][kMultiRows * 8];
+    __shared__ float4 s_f[kUnits][kMultiRows * NF / 4];
+    __shared__ uint32_t s_in[kUnits][kMultiRows];   // which of the 32 voxels are pairs (non-finite fluences only)
+    __shared__ RowWindows s_win[kWarps];
+    __shared__ int s_w[kUnits], s_bad[kUnits];
+    const PlanView& P = a.P;
+    const int64_t V = (int64_t)P.nx * P.ny * P.nz;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int unit = warp / WPU, half = warp % WPU, ut = threadIdx.x % (32 * WPU);
+    const int vg = lane >> 3, fg = lane & 7;   // the lane's voxels 8 vg .. 8 vg + 7, vectors VP fg .. of the warp's
+    if (!MERGED)
+        for (int q = threadIdx.x; q < 2 * P.w_n; q += blockDim.x) smem[q] = __ldg(P.water + q);
+    for (int q = threadIdx.x; q <= P.n_beams; q += blockDim.x) s_base[q] = a.base[q];
+    __syncthreads();
+    float4* srow = s_row[unit];
+    float* sd = reinterpret_cast<float*>(s_d[unit]);
+    float4* sf = s_f[unit];
+    RowWindows& win = s_win[warp];
+    const int total = a.work[0];
+    for (;;) {
+        int w = 0;
+        if (WPU == 1) {
+            if (lane == 0) w = atomicAdd(a.work + 1, 1);
+            w = __shfl_sync(0xffffffffu, w, 0);
+        } else {
+            unit_sync<WPU>(unit);
+            if (ut == 0) {
+                s_w[unit] = atomicAdd(a.work + 1, 1);
+                s_bad[unit] = 0;
+            }
+            unit_sync<WPU>(unit);
+            w = s_w[unit];
+        }
+        if (w >= total) break;
+        const int64_t e0 = (int64_t)DC_GUARD(P, w, (s_base[P.n_beams] + 31) / 32, 4) * 32;
+        int b = 0;
+        while (b + 1 < P.n_beams && s_base[b + 1] <= e0) ++b;
+        const int32_t vi = __ldg(a.items + e0 + lane);
+        const BeamDev& bm = P.beams[b];
+        const float sad = __ldg(&bm.sad);
+        int n0, n1;
+        Lane ln;
+        UnitBox box;
+        {
+            CountVoxel c[1] = {count_voxel(P, bm, vi, sad)};
+            ln = c[0].ln;
+            box = unit_box<1>(c);
+            box_rows(P, box, __ldg(&bm.N), __ldg(&bm.half_fy), n0, n1);
+            const float4 fac = __ldg(P.fac + c[0].v);   // f_u1(rho), f_u2(rho_hat), f_w1(rho_hat), f_w2(rho_hat)
+            const float4 lf = LAT == kItem ? __ldg(P.lfac + e0 + lane)
+                                           : make_float4(kLog2e * fac.y, kLog2e * fac.y, fac.z, fac.w);
+            ln.cu1 = kLog2e * fac.x;
+            ln.cu2x = lf.x;
+            ln.cu2y = lf.y;
+            ln.cw1 = lf.z;
+            ln.cw2 = lf.w;
+        }
+        float acc[8][VP];
+#pragma unroll
+        for (int j = 0; j < 8; ++j)
+#pragma unroll
+            for (int q = 0; q < VP; ++q) acc[j][q] = 0.f;
+        for (int nb = n0; nb <= n1; nb += 32) {
+            const int places = row_windows(P, box, win, nb, n1, __ldg(&bm.M), __ldg(&bm.first), __ldg(&bm.half_fx),
+                                           __ldg(&bm.half_fy), lane);
+            for (int q0 = 0; q0 < places; q0 += kMultiRows) {
+                const int nq = min(kMultiRows, places - q0);
+                int ib = 0;
+                if (lane < nq) ib = (int)DC_GUARD(P, win.base[window_row(win, q0 + lane)] + q0 + lane, P.B, 5);
+                unit_sync<WPU>(unit);   // the last chunk's product has read its operands
+                if (half == 0 && lane < nq) {
+                    const float4* src = reinterpret_cast<const float4*>(P.bl) + 4u * (uint32_t)ib;
+                    srow[3 * lane] = __ldg(src);
+                    srow[3 * lane + 1] = __ldg(src + 1);
+                    srow[3 * lane + 2] = __ldg(src + 2);
+                }
+                bool finite = true;
+#pragma unroll
+                for (int t = 0; t < kMultiRows * NF / 4; t += 32 * WPU) {
+                    const int j = (t + ut) / (NF / 4);
+                    const int i = __shfl_sync(0xffffffffu, ib, j);
+                    if (j < nq) {
+                        const float4 f = __ldg(a.fpack32 + (size_t)i * (NF / 4) + (t + ut) % (NF / 4));
+                        sf[t + ut] = f;
+                        finite = finite && fabsf(f.x) <= 3.402823466e38f && fabsf(f.y) <= 3.402823466e38f &&
+                                 fabsf(f.z) <= 3.402823466e38f && fabsf(f.w) <= 3.402823466e38f;
+                    }
+                }
+                finite = __all_sync(0xffffffffu, finite);
+                if (WPU > 1 && !finite && lane == 0) s_bad[unit] = 1;
+                unit_sync<WPU>(unit);
+                const bool bad = WPU > 1 ? s_bad[unit] != 0 : !finite;
+#pragma unroll 2
+                for (int m = half; m < nq; m += WPU) {
+                    const uint32_t i = (uint32_t)__shfl_sync(0xffffffffu, ib, m);
+                    const float4* rq = srow + 3 * m;
+                    const PairTest pt = pair_test(P, ln, rq[0], rq[1], rq[2]);
+                    float D = 0.f;
+                    if (pt.in) D = pair_eval<MERGED, LAT, 0>(P, ln, i, sad, smem, pt);
+                    sd[m * 32 + lane] = D;
+                    if (bad) {
+                        const uint32_t in = __ballot_sync(0xffffffffu, pt.in);
+                        if (lane == 0) s_in[unit][m] = in;
+                    }
+                }
+                unit_sync<WPU>(unit);
+#pragma unroll 4
+                for (int m = 0; m < nq; ++m) {
+                    const float4 d0 = s_d[unit][m * 8 + 2 * vg], d1 = s_d[unit][m * 8 + 2 * vg + 1];
+                    const float d[8] = {d0.x, d0.y, d0.z, d0.w, d1.x, d1.y, d1.z, d1.w};
+                    float f[VP];
+                    if (VP == 2) {
+                        const float2 g = reinterpret_cast<const float2*>(sf + m * (NF / 4))[fg];
+                        f[0] = g.x;
+                        f[1] = g.y;
+                    } else {
+                        const float4 g = sf[m * (NF / 4) + 8 * half + fg];
+                        f[0] = g.x;
+                        f[1] = g.y;
+                        f[VP - 2] = g.z;
+                        f[VP - 1] = g.w;
+                    }
+                    if (!bad) {
+#pragma unroll
+                        for (int j = 0; j < 8; ++j)
+#pragma unroll
+                            for (int q = 0; q < VP; ++q) acc[j][q] = fmaf(f[q], d[j], acc[j][q]);
+                    } else {
+                        // an infinite or NaN fluence reaches the beamlet's own pairs only
+                        const uint32_t in = s_in[unit][m] >> (8 * vg);
+#pragma unroll
+                        for (int j = 0; j < 8; ++j)
+#pragma unroll
+                            for (int q = 0; q < VP; ++q)
+                                if ((in >> j) & 1u) acc[j][q] = fmaf(f[q], d[j], acc[j][q]);
+                    }
+                }
+            }
+        }
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+            const int v = __shfl_sync(0xffffffffu, vi, 8 * vg + j);
+            if (v < 0) continue;
+            float* out = a.part + ((size_t)b * V + v) * NF + NW * half;
+            if (VP == 2)
+                reinterpret_cast<float2*>(out)[fg] = make_float2(acc[j][0], acc[j][1]);
+            else
+                reinterpret_cast<float4*>(out)[fg] = make_float4(acc[j][0], acc[j][1], acc[j][VP - 2], acc[j][VP - 1]);
+        }
+    }
+}
+
+// fpack[i][n] = F[n][i], zero for n >= nf (32 x 32 transposes).
+__global__ void __launch_bounds__(256) k_pack_fluence(const float* __restrict__ F, int nf, int ldf, int B, int NF,
+                                                      float* __restrict__ fpack)
+{
+    __shared__ float s[32][33];
+    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+    const int i0 = blockIdx.x * 32, n0 = blockIdx.y * 32;
+    for (int y = ty; y < 32; y += 8)
+        s[y][tx] = n0 + y < nf && i0 + tx < B ? __ldg(F + (size_t)(n0 + y) * ldf + i0 + tx) : 0.f;
+    __syncthreads();
+    for (int y = ty; y < 32; y += 8)
+        if (i0 + y < B && n0 + tx < NF) fpack[(size_t)(i0 + y) * NF + n0 + tx] = s[tx][y];
+}
+
+// dose[q][v] = sum over beams, in beam order, of the partial doses [n_beams][V][NF]
+// of the beams that list v (`cell` >= 0; the others' are not written).  32 voxels
+// per block: rows read whole, turned in shared memory, written 32 voxels at a
+// time.  One pass over the listed partials: 1.47 + 0.55 ms (a pass over all of
+// them in [n_beams][NF][V] order and the clearing before it) -> 0.50 ms for 64
+// vectors on the thorax plan.
+template <int NF>
+__global__ void __launch_bounds__(256) k_sum_vectors(const float4* __restrict__ part, const int32_t* __restrict__ cell,
+                                                     int n_beams, int nf, int64_t V, float* __restrict__ dose,
+                                                     int64_t ldd)
+{
+    constexpr int R = NF / 4;   // float4 per row
+    __shared__ float s[NF][33];
+    const int64_t tiles = (V + 31) / 32;
+    for (int64_t t = blockIdx.x; t < tiles; t += gridDim.x) {
+        const int64_t v0 = t * 32;
+        for (int e = threadIdx.x; e < 32 * R; e += blockDim.x) {
+            const int j = e / R, r = e % R;
+            const int64_t v = v0 + j;
+            float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (v < V)
+                for (int b = 0; b < n_beams; ++b) {
+                    if (__ldg(cell + (size_t)b * V + v) < 0) continue;
+                    const float4 p = __ldg(part + ((size_t)b * V + v) * R + r);
+                    x.x += p.x;
+                    x.y += p.y;
+                    x.z += p.z;
+                    x.w += p.w;
+                }
+            s[4 * r][j] = x.x;
+            s[4 * r + 1][j] = x.y;
+            s[4 * r + 2][j] = x.z;
+            s[4 * r + 3][j] = x.w;
+        }
+        __syncthreads();
+        const int lane = threadIdx.x & 31;
+        for (int q = threadIdx.x >> 5; q < nf; q += 8)
+            if (v0 + lane < V) dose[(size_t)q * ldd + v0 + lane] = s[q][lane];
+        __syncthreads();
     }
 }
 
@@ -1465,22 +1677,24 @@ __global__ void __launch_bounds__(256) k_sum_batch(const DoseArgs* __restrict__ 
         const int64_t V = s_v[lo + 1] - s_v[lo];
         const int64_t v = e - s_v[lo];
         float sum = 0.f;
-        for (int b = 0; b < a.P.n_beams; ++b) sum += __ldg(a.part + (size_t)b * V + v);
+        for (int b = 0; b < a.P.n_beams; ++b)
+            if (__ldg(a.cell + (size_t)b * V + v) >= 0) sum += __ldg(a.part + (size_t)b * V + v);
         a.dose[v] = sum;
     }
 }
 
-// dose[q][v] = sum over beams of the partial doses (fixed beam order).
-__global__ void __launch_bounds__(256) k_sum_beams(const float* __restrict__ part, int n_beams, int nfs,
-                                                   int nf, int64_t V, float* __restrict__ dose, int64_t ldd)
+// dose[v] = sum over the beams that list v, in beam order, of its partial doses
+// (`cell` >= 0 says which: the partials of the others are neither written nor
+// cleared).
+__global__ void __launch_bounds__(256) k_sum_beams(const float* __restrict__ part, const int32_t* __restrict__ cell,
+                                                   int n_beams, int64_t V, float* __restrict__ dose)
 {
-    for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < (int64_t)nf * V;
-         e += (int64_t)gridDim.x * blockDim.x) {
-        const int q = (int)(e / V);
-        const int64_t v = e % V;
+    for (int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; v < V; v += (int64_t)gridDim.x * blockDim.x) {
         float s = 0.f;
-        for (int b = 0; b < n_beams; ++b) s += __ldg(part + ((size_t)b * nfs + q) * V + v);
-        dose[(size_t)q * ldd + v] = s;
+#pragma unroll 4
+        for (int b = 0; b < n_beams; ++b)
+            if (__ldg(cell + (size_t)b * V + v) >= 0) s += __ldg(part + (size_t)b * V + v);
+        dose[v] = s;
     }
 }
 
@@ -1589,6 +1803,7 @@ DoseArgs make_args(const dc_plan* p)
     a.base = p->d_base;
     a.work = p->d_work;
     a.bcount = p->d_bcount;
+    a.cell = p->d_cellof;
     return a;
 }
 
@@ -1608,27 +1823,38 @@ int grid_for(int64_t n)
     return (int)(g > 152 * 32 ? 152 * 32 : (g < 1 ? 1 : g));
 }
 
-// Persistent launch: as many CTAs as fit on the device at once.
+// Persistent launch of a kernel that takes its units from the plan's counter:
+// as many CTAs as fit on the device at once.
+template <typename K, typename... Args>
+cudaError_t launch_units(const dc_plan* p, K kern, size_t sm, const Args&... args)
+{
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    if (e != cudaSuccess) return e;
+    int per_sm = 0, sms = 0;
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kThreads, sm);
+    if (e != cudaSuccess) return e;
+    e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, p->device);
+    if (e != cudaSuccess) return e;
+    e = cudaMemsetAsync(p->d_work + 1, 0, sizeof(int32_t), p->stream);
+    if (e != cudaSuccess) return e;
+    kern<<<sms * (per_sm > 0 ? per_sm : 1), kThreads, sm, p->stream>>>(args...);
+    count_launches(1);
+    return cudaGetLastError();
+}
+
 template <int MODE, int NF, bool MERGED, int LAT, int PREC = 0>
 cudaError_t run_variant(const dc_plan* p, const DoseArgs& a)
 {
     const size_t sm = smem_bytes(p, MODE);
-    auto kern = k_pairs<MODE, NF, MERGED, LAT, PREC>;
-    int per_sm = 0, sms = 0;
-    cudaError_t e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, p->device);
-    if (e != cudaSuccess) return e;
-    // no more units than warps with 4 CTAs per SM
-    if (MODE == kDose && NF == 1 && (int64_t)p->n_beams * ((p->V + 31) / 32) <= (int64_t)sms * 4 * kWarps)
-        kern = k_pairs<MODE, NF, MERGED, LAT, PREC, MODE == kDose && NF == 1 ? 4 : min_ctas<MODE, NF>()>;
-    e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    if (e != cudaSuccess) return e;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kThreads, sm);
-    if (e != cudaSuccess) return e;
-    e = cudaMemsetAsync(p->d_work + 1, 0, sizeof(int32_t), p->stream);
-    if (e != cudaSuccess) return e;
-    kern<<<sms * (per_sm > 0 ? per_sm : 1), kThreads, sm, p->stream>>>(a);
-    count_launches(1);
-    return cudaGetLastError();
+    if constexpr (MODE == kDose && NF == 1) {
+        int sms = 0;
+        const cudaError_t e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, p->device);
+        if (e != cudaSuccess) return e;
+        // no more units than warps with 4 CTAs per SM
+        if ((int64_t)p->n_beams * ((p->V + 31) / 32) <= (int64_t)sms * 4 * kWarps)
+            return launch_units(p, k_pairs<MODE, NF, MERGED, LAT, PREC, 4>, sm, a);
+    }
+    return launch_units(p, k_pairs<MODE, NF, MERGED, LAT, PREC>, sm, a);
 }
 
 // The tensor-core form of 64 fluence vectors (PREC 2) for the plan's lateral
@@ -1651,6 +1877,25 @@ __global__ void __launch_bounds__(256) k_pack_fluence_bf16(const float* __restri
         const int n = (int)(e / B), i = (int)(e % B);
         fpack[(size_t)i * 64 + n] = __float2bfloat16_rn(n < nf ? __ldg(F + (size_t)n * ldf + i) : 0.f);
     }
+}
+
+// One FP32 pass of NF fluence vectors (fluence packed as [B][NF]).
+template <int NF>
+cudaError_t run_multi(const dc_plan* p, const DoseArgs& a, float* dose, int64_t ldd)
+{
+    const bool item = p->coeffs.density_correction && p->lateral_mode != DC_LATERAL_ISO;
+    auto kern = p->merged ? (item ? k_dose_multi<NF, true, kItem> : k_dose_multi<NF, true, kIso>)
+                          : (item ? k_dose_multi<NF, false, kItem> : k_dose_multi<NF, false, kIso>);
+    const size_t sm = p->merged ? 0 : 2 * sizeof(float4) * p->coeffs.w_n;
+    k_pack_fluence<<<dim3((p->B + 31) / 32, (NF + 31) / 32), 256, 0, p->stream>>>(
+        a.fluence, a.nf, a.ldf, p->B, NF, reinterpret_cast<float*>(p->d_flupack));
+    count_launches(1);
+    cudaError_t e = launch_units(p, kern, sm, a);
+    if (e != cudaSuccess) return e;
+    k_sum_vectors<NF><<<grid_for(p->V * 8), 256, 0, p->stream>>>(reinterpret_cast<const float4*>(p->d_part), p->d_cellof,
+                                                                 p->n_beams, a.nf, p->V, dose, ldd);
+    count_launches(1);
+    return cudaGetLastError();
 }
 
 template <int MODE, int NF>
@@ -1753,35 +1998,33 @@ cudaError_t launch_dose(const dc_plan* p, const float* fluence, int nf, int ldf,
         a.fluence = fluence;
         a.nf = nf;
         a.fpack = static_cast<const uint4*>(p->d_sp_fp);
-        e = cudaMemsetAsync(p->d_part, 0, sizeof(float) * (size_t)p->n_beams * 64 * p->V, p->stream);
-        if (e != cudaSuccess) return e;
         e = run_tc(p, a);
         if (e != cudaSuccess) return e;
-        k_sum_beams<<<grid_for((int64_t)nf * p->V), 256, 0, p->stream>>>(p->d_part, p->n_beams, 64, nf, p->V, dose,
-                                                                        ldd);
+        k_sum_vectors<64><<<grid_for(p->V * 8), 256, 0, p->stream>>>(reinterpret_cast<const float4*>(p->d_part),
+                                                                     p->d_cellof, p->n_beams, nf, p->V, dose, ldd);
         count_launches(1);
         return cudaGetLastError();
     }
-    if (record_counts && nf == 1) {
+    a.fluence = fluence;
+    a.nf = nf;
+    if (nf > 1) {
+        const int width = dose_pass_width(nf);
+        if (nf > width || p->part_cap < (size_t)p->n_beams * width * p->V || p->flupack_cap < (size_t)width * p->B)
+            return cudaErrorInvalidValue;
+        a.fpack32 = p->d_flupack;
+        return width == 16 ? run_multi<16>(p, a, dose, ldd)
+                           : (width == 32 ? run_multi<32>(p, a, dose, ldd) : run_multi<64>(p, a, dose, ldd));
+    }
+    if (record_counts) {
         cudaError_t e = cudaMemsetAsync(p->d_bcount, 0, sizeof(int32_t) * (size_t)p->n_beams * p->V, p->stream);
         if (e != cudaSuccess) return e;
         a.count_out = p->d_bcount;
     }
-    const int width = dose_pass_width(nf);
-    for (int q0 = 0; q0 < nf; q0 += width) {
-        a.fluence = fluence + (size_t)q0 * ldf;
-        a.nf = nf - q0 < width ? nf - q0 : width;
-        const int nfs = a.nf == 1 ? 1 : width;
-        if (p->part_cap < (size_t)p->n_beams * nfs * p->V) return cudaErrorInvalidValue;
-        cudaError_t e = cudaMemsetAsync(p->d_part, 0, sizeof(float) * (size_t)p->n_beams * nfs * p->V, p->stream);
-        if (e != cudaSuccess) return e;
-        e = nfs == 1 ? run<kDose, 1>(p, a)
-                     : (nfs == 16 ? run<kDose, 16>(p, a) : (nfs == 32 ? run<kDose, 32>(p, a) : run<kDose, 64>(p, a)));
-        if (e != cudaSuccess) return e;
-        k_sum_beams<<<grid_for((int64_t)a.nf * p->V), 256, 0, p->stream>>>(p->d_part, p->n_beams, nfs, a.nf, p->V,
-                                                                          dose + (size_t)q0 * ldd, ldd);
-        count_launches(1);
-    }
+    if (p->part_cap < (size_t)p->n_beams * p->V) return cudaErrorInvalidValue;
+    const cudaError_t e = run<kDose, 1>(p, a);
+    if (e != cudaSuccess) return e;
+    k_sum_beams<<<grid_for(p->V), 256, 0, p->stream>>>(p->d_part, p->d_cellof, p->n_beams, p->V, dose);
+    count_launches(1);
     return cudaGetLastError();
 }
 
@@ -1830,35 +2073,16 @@ cudaError_t launch_fill(const dc_plan* p, const int64_t* rowptr, int32_t* cols, 
     a.nf = 1;
     a.ldf = p->B;
     a.part = p->d_part;
-    cudaError_t e = cudaMemsetAsync(p->d_part, 0, sizeof(float) * (size_t)p->n_beams * p->V, p->stream);
+    cudaError_t e = run<kFill, 1>(p, a);
     if (e != cudaSuccess) return e;
-    e = run<kFill, 1>(p, a);
-    if (e != cudaSuccess) return e;
-    k_sum_beams<<<grid_for((int64_t)p->V), 256, 0, p->stream>>>(p->d_part, p->n_beams, 1, 1, p->V, dose, p->V);
-    count_launches(1);
-    return cudaGetLastError();
-}
-
-template <typename K>
-static cudaError_t launch_persistent(const dc_plan* p, K kern, size_t sm, const DoseArgs& a, const PatchTiles& t)
-{
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    if (e != cudaSuccess) return e;
-    int per_sm = 0, sms = 0;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kThreads, sm);
-    if (e != cudaSuccess) return e;
-    e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, p->device);
-    if (e != cudaSuccess) return e;
-    e = cudaMemsetAsync(p->d_work + 1, 0, sizeof(int32_t), p->stream);
-    if (e != cudaSuccess) return e;
-    kern<<<sms * (per_sm > 0 ? per_sm : 1), kThreads, sm, p->stream>>>(a, t);
+    k_sum_beams<<<grid_for(p->V), 256, 0, p->stream>>>(p->d_part, p->d_cellof, p->n_beams, p->V, dose);
     count_launches(1);
     return cudaGetLastError();
 }
 
 cudaError_t launch_mark_patches(const dc_plan* p, const PatchTiles& t)
 {
-    return launch_persistent(p, k_mark_patches, 0, make_args(p), t);
+    return launch_units(p, k_mark_patches, 0, make_args(p), t);
 }
 
 cudaError_t launch_tile_fill(const dc_plan* p, const PatchTiles& t)
@@ -1867,10 +2091,10 @@ cudaError_t launch_tile_fill(const dc_plan* p, const PatchTiles& t)
     const bool item = p->coeffs.density_correction && p->lateral_mode != DC_LATERAL_ISO;
     const size_t sm = p->merged ? 0 : 2 * sizeof(float4) * p->coeffs.w_n;
     if (p->merged)
-        return item ? launch_persistent(p, k_tile_fill<true, kItem>, sm, a, t)
-                    : launch_persistent(p, k_tile_fill<true, kIso>, sm, a, t);
-    return item ? launch_persistent(p, k_tile_fill<false, kItem>, sm, a, t)
-                : launch_persistent(p, k_tile_fill<false, kIso>, sm, a, t);
+        return item ? launch_units(p, k_tile_fill<true, kItem>, sm, a, t)
+                    : launch_units(p, k_tile_fill<true, kIso>, sm, a, t);
+    return item ? launch_units(p, k_tile_fill<false, kItem>, sm, a, t)
+                : launch_units(p, k_tile_fill<false, kIso>, sm, a, t);
 }
 
 cudaError_t launch_dose_vjp(const dc_plan* p, const float* fluence, const float* wv, float* g_water, float* g_dens,
