@@ -210,6 +210,8 @@ static void bin_geometry(dc_plan* p, float tile, float slab)
         BinGeom G;
         G.tile = tile;
         G.slab = slab;
+        G.inv_tile = 1.0f / tile;
+        G.inv_slab = 1.0f / slab;
         G.rw_max = (float)(p->coeffs.roi_radius * (sad / zmin) * inv_cos * 1.001 + 2e-3);
         const double ea = hfx + G.rw_max + tile, ec = hfy + G.rw_max + tile;
         G.a0 = (float)-ea;
@@ -306,12 +308,12 @@ static dc_status check_inputs(const float* ct, const dc_grid* g, const dc_beam* 
     return DC_OK;
 }
 
-// Algorithm A1 steps 1-6 on the plan's stream for the density in d_rho.
+// The density-dependent part of Algorithm A1 steps 1-6 on the plan's stream for
+// the density in d_rho (the beamlet geometry of steps 2-3 is the plan's).
 static dc_status rerun_density_steps(dc_plan* p)
 {
-    DC_CUDA(launch_smooth(p, p->coeffs.smooth_sigma));
-    DC_CUDA(launch_factors(p));
-    DC_CUDA(launch_beamlets(p));
+    DC_CUDA(launch_smooth_factors(p));
+    DC_CUDA(launch_trace(p));
     DC_CUDA(launch_binning(p));
     if (p->coeffs.density_correction && p->lateral_mode != DC_LATERAL_ISO) DC_CUDA(launch_lateral(p));
     p->pairs = -1;
@@ -390,7 +392,7 @@ static dc_status create_impl(dc_plan* p, const float* ct, uint32_t flags)
     DC_CUDA(dalloc(&p->d_beamin, p->n_beams));
     DC_CUDA(dalloc(&p->d_bl, p->B));
     DC_CUDA(dalloc(&p->d_theta, p->B));
-    DC_CUDA(dalloc(&p->d_ray, 8 * (size_t)p->B));
+    DC_CUDA(dalloc(&p->d_ray, 12 * (size_t)p->B));
     DC_CUDA(dalloc(&p->d_lio, p->B));
     DC_CUDA(dalloc(&p->d_tab, 2 * (size_t)p->B * p->Kmax));
     DC_CUDA(dalloc(&p->d_arow, (size_t)p->B * c.a_nt));
@@ -438,6 +440,7 @@ static dc_status create_impl(dc_plan* p, const float* ct, uint32_t flags)
                             cudaMemcpyHostToDevice, p->stream));
     DC_CUDA(cudaMemcpyAsync(p->d_beamin, p->beams.data(), sizeof(dc_beam) * p->n_beams,
                             cudaMemcpyHostToDevice, p->stream));
+    DC_CUDA(launch_geometry(p));
     dc_status s = compute_density_steps(p, ct, flags);
     if (s != DC_OK) return s;
     DC_CUDA(cudaStreamSynchronize(p->stream));

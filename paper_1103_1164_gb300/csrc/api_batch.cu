@@ -122,9 +122,8 @@ cudaError_t enqueue(dc_batch* bt, bool density)
             // the plan's launchers enqueue on p->stream: point it at the branch
             cudaStream_t own = p->stream;
             p->stream = br;
-            e = launch_smooth(p, p->coeffs.smooth_sigma);
-            if (e == cudaSuccess) e = launch_factors(p);
-            if (e == cudaSuccess) e = launch_beamlets(p);
+            e = launch_smooth_factors(p);
+            if (e == cudaSuccess) e = launch_trace(p);
             if (e == cudaSuccess) e = launch_binning(p);
             if (e == cudaSuccess && p->coeffs.density_correction && p->lateral_mode != DC_LATERAL_ISO)
                 e = launch_lateral(p);

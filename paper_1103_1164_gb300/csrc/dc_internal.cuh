@@ -33,7 +33,7 @@ struct dc_plan {
     dc::BeamDev* d_beams = nullptr;
     dc::BeamletDev* d_bl = nullptr;
     float* d_theta = nullptr;
-    double* d_ray = nullptr;         // [B][8]: FP64 source (3) and direction (3) of each beamlet axis
+    double* d_ray = nullptr;         // [B][12]: FP64 axis of each beamlet (see k_beamlets)
     float2* d_lio = nullptr;         // [B]: (L_in, L_out) of each axis, L_out < 0 if it misses the body
     float4* d_tab = nullptr;
     float2* d_arow = nullptr;
@@ -193,9 +193,9 @@ dc_status cuda_fail(cudaError_t e, const char* what);
     } while (0)
 
 // kernel launchers (defined in the kernel translation units) ------------------
-cudaError_t launch_smooth(const dc_plan* p, float sigma);
-cudaError_t launch_factors(const dc_plan* p);
-cudaError_t launch_beamlets(const dc_plan* p);   // also builds the theta-blended A rows
+cudaError_t launch_geometry(const dc_plan* p);         // once per plan: beamlet geometry, theta-blended A rows
+cudaError_t launch_smooth_factors(const dc_plan* p);   // smoothed density and the voxels' factors
+cudaError_t launch_trace(const dc_plan* p);            // body entry and exit, depth tables
 cudaError_t launch_binning(const dc_plan* p);
 // record_counts (one fluence vector only): the pass also writes the per-beam
 // pair counts that launch_count would (the matrix pattern then needs no

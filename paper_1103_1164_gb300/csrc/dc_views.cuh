@@ -34,7 +34,7 @@ struct BeamletDev {
 // in the isocentre plane starting at (a0, c0), depth slabs of `slab` cm
 // starting at zz0; cell = (tc * nta + ta) * nzs + slab index.
 struct BinGeom {
-    float a0, c0, tile, zz0, slab, rw_max;
+    float a0, c0, tile, zz0, slab, rw_max, inv_tile, inv_slab;
     int nta, ntc, nzs, cells;
 };
 

@@ -340,7 +340,7 @@ __device__ __forceinline__ void pair_grad(const PlanView& P, const float4 facv, 
 }
 
 // The interpolation of a density-function table at density r (clamped to
-// its domain), as k_factors reads it: entry j with weight 1 - w, j + 1 with w.
+// its domain), as voxel_factors reads it: entry j with weight 1 - w, j + 1 with w.
 __device__ __forceinline__ void dens_bins(const PlanView& P, float r, int& j, float& w)
 {
     const float sx = fminf(fmaxf((r - P.f_rho0) * P.inv_drho, 0.f), (float)(P.f_n - 1));
