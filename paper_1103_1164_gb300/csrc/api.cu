@@ -122,7 +122,8 @@ static void free_plan(dc_plan* p)
                     p->d_bin, p->d_bounds, p->d_cellof, p->d_hist, p->d_nitems, p->d_bstart, p->d_bscan,
                     p->d_base, p->d_work,
                     p->d_items, p->d_part, p->d_bcount, p->d_sp_fp, p->d_sp_p, p->d_err,
-                    p->d_flupack, p->d_lfac, p->d_mlp_frag, p->d_mlp_bias, p->d_nfall, p->d_leaf, p->d_chk, p->d_grad};
+                    p->d_flupack, p->d_lfac, p->d_quad, p->d_mlp_frag, p->d_mlp_bias, p->d_nfall, p->d_leaf,
+                    p->d_chk, p->d_grad};
     for (void* b : bufs)
         if (b) cudaFree(b);
     p->spmm_free();
@@ -428,6 +429,7 @@ static dc_status create_impl(dc_plan* p, const float* ct, uint32_t flags)
     p->part_cap = nb * V;
     DC_CUDA(dalloc(&p->d_bcount, nb * V));
     DC_CUDA(dalloc(&p->d_lfac, nb * (V + 32)));
+    DC_CUDA(dalloc(&p->d_quad, V));
     DC_CUDA(dalloc(&p->d_nfall, 1));
     DC_CUDA(dalloc(&p->d_chk, 1));
     DC_CUDA(cudaMemsetAsync(p->d_chk, 0, sizeof(int32_t), p->stream));

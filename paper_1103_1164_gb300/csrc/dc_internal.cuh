@@ -43,6 +43,7 @@ struct dc_plan {
     int lateral_mode = 0;
     int precision = DC_PRECISION_FP32;   // arithmetic of the direct dose (dc_fspb_set_precision)
     float4* d_lfac = nullptr;        // [n_beams][V + 32]
+    float4* d_quad = nullptr;        // [V] density at a voxel and its +x, +y neighbours (axis stencil)
     float* d_leaf = nullptr;         // leaf sequences of dc_fluence_from_leaves (packed)
     size_t leaf_cap = 0;             // floats allocated at d_leaf
     uint2* d_mlp_frag = nullptr;     // BF16 B fragments of the surrogate network
