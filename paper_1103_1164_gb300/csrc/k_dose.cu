@@ -40,6 +40,11 @@ constexpr int kRingLd = kRing + 1;
 constexpr int row_max(int mode, int nf = 1) { return mode == 2 || nf > 32 ? 16 : 32; }
 
 enum Mode { kDose = 0, kCount = 1, kFill = 2, kGrad = 3 };
+// work items per unit of the backward pass, whose phantoms have few units (a 60^3
+// grid: 6,750 for 4,864 warps, so whole units ran in two rounds).  A single call on
+// that grid: 385 us with 1 item, 254 with 2, 200 with 4, 220 with 8; 30^3: 225, 156,
+// 121, 106; 72^3, two beams: 390, 300, 267, 283.
+constexpr int kGradSplit = 4;
 
 // PREC 2, the tensor-core form of the multi-fluence dose (64 vectors): per
 // warp and chunk of 16 beamlets, Y[32 voxels][64] += D[32][16] F[16][64] as
@@ -272,9 +277,73 @@ __device__ __forceinline__ void penumbra_du(float ax, float u, float x0, float& 
     dp = 0.5f * (fmaf(-dd, e1, 0.f) + (ax + x0) * e2);
 }
 
+// The backward pass's sums for the two samples around depth t, j and j + 1, of
+// the water tables u_1^w, u_2^w, omega_1^w, omega_2^w.  A voxel's depth changes
+// little from one beamlet to the next, so a lane keeps the sums of its current
+// segment in registers and adds them to the CTA's bins when the segment changes:
+// with eight shared-memory atomics per pair, contended by the lanes of a warp
+// (whose depths span a few samples), they were what bound the kernel: a call on a
+// 60^3 slab (7.5 M pairs) took 652 us, now 160, kGradSplit included.
+struct WaterSums {
+    int j;
+    float a0[4], a1[4];
+};
+
+__device__ __forceinline__ void flush_water(WaterSums& w, float* sgw, int wn)
+{
+    if (w.j >= 0) {
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            atomicAdd(sgw + q * wn + w.j, w.a0[q]);
+            if (w.j + 1 < wn) atomicAdd(sgw + q * wn + w.j + 1, w.a1[q]);
+        }
+    }
+#pragma unroll
+    for (int q = 0; q < 4; ++q) w.a0[q] = w.a1[q] = 0.f;
+}
+
+// Adds the lanes' eight values to the bins bin(key, q): the lanes of a warp mostly
+// share a few keys (depth segments, densities of a tissue), so the sum over a key's
+// lanes is formed in registers, a value per four lanes, before one atomic each; a
+// shared-memory FP32 atomic is a compare-and-swap loop, 32 rounds for 32 lanes in
+// one bin.  Lanes of a fifth and later keys add their values themselves.  Two beams
+// on a mixed 72^3 body: 305 -> 267 us, the 60^3 slab 210 -> 202 (single calls).
+template <typename Bin>
+__device__ __forceinline__ void add_by_key(int key, bool on, const float (&v)[8], int lane, Bin&& bin)
+{
+    uint32_t todo = __ballot_sync(0xffffffffu, on);
+    for (int g = 0; g < 4 && todo; ++g) {
+        const int k = __shfl_sync(0xffffffffu, key, __ffs(todo) - 1);
+        const bool mine = on && key == k;
+        todo &= ~__ballot_sync(0xffffffffu, mine);
+        float x[4], y[2], z;
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const float lo = mine ? v[q] : 0.f, hi = mine ? v[q + 4] : 0.f;
+            x[q] = (lane & 16 ? hi : lo) + __shfl_xor_sync(0xffffffffu, lane & 16 ? lo : hi, 16);
+        }
+#pragma unroll
+        for (int q = 0; q < 2; ++q)
+            y[q] = (lane & 8 ? x[q + 2] : x[q]) + __shfl_xor_sync(0xffffffffu, lane & 8 ? x[q] : x[q + 2], 8);
+        z = (lane & 4 ? y[1] : y[0]) + __shfl_xor_sync(0xffffffffu, lane & 4 ? y[0] : y[1], 4);
+        z += __shfl_xor_sync(0xffffffffu, z, 2);
+        z += __shfl_xor_sync(0xffffffffu, z, 1);
+        if ((lane & 3) == 0) {
+            float* p = bin(k, (lane >> 4) * 4 + (lane >> 3 & 1) * 2 + (lane >> 2 & 1));
+            if (p) atomicAdd(p, z);
+        }
+    }
+    if (todo >> lane & 1)
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {
+            float* p = bin(key, q);
+            if (p) atomicAdd(p, v[q]);
+        }
+}
+
 // Backward pass of one pair (commissioning fit, Section 2.1): with
-// c = w_v f_i, accumulates c dD_i(r)/d(entry) into the shared bins of the
-// water tables u_1^w, u_2^w, omega_1^w, omega_2^w (the two samples around t);
+// c = w_v f_i, accumulates c dD_i(r)/d(entry) into the lane's water-table sums
+// (the two samples around t);
 // into the lane's per-voxel sums the derivatives with respect to the values
 // f_u1(rho), f_u2(rho_hat), f_omega1(rho_hat), f_omega2(rho_hat) (scattered to
 // the density-function bins once per work unit); and into gc the derivatives
@@ -282,7 +351,7 @@ __device__ __forceinline__ void penumbra_du(float ax, float u, float x0, float& 
 // Paper's lateral form, general (unmerged) tables, density correction on.
 __device__ __forceinline__ void pair_grad(const PlanView& P, const float4 facv, const uint32_t i, const float sad,
                                           const float4* __restrict__ sW, const PairTest& pt, const float c,
-                                          float* sgw, float gl[4], float gc[2])
+                                          float* sgw, WaterSums& ws, float gl[4], float gc[2])
 {
     const float L = pt.L;
     const float t = L - pt.L_in;
@@ -319,17 +388,16 @@ __device__ __forceinline__ void pair_grad(const PlanView& P, const float4 facv, 
     const float g_u1 = K * om1 * fmaf(d1x, p1y, p1x * d1y);  // dD/d u_1
     const float g_u2 = K * om2 * fmaf(d2x, p2y, p2x * d2y);
     // water tables: val = w[jw] + fw (w[jw + 1] - w[jw])
-    const int wn = P.w_n;
+    if (jw != ws.j) {
+        flush_water(ws, sgw, P.w_n);
+        ws.j = jw;
+    }
     const float a0 = 1.f - fw;
-    atomicAdd(sgw + 0 * wn + jw, a0 * g_u1 * facv.x);
-    atomicAdd(sgw + 1 * wn + jw, a0 * g_u2 * facv.y);
-    atomicAdd(sgw + 2 * wn + jw, a0 * g_om1 * facv.z);
-    atomicAdd(sgw + 3 * wn + jw, a0 * g_om2 * facv.w);
-    if (jw + 1 < wn && fw != 0.f) {
-        atomicAdd(sgw + 0 * wn + jw + 1, fw * g_u1 * facv.x);
-        atomicAdd(sgw + 1 * wn + jw + 1, fw * g_u2 * facv.y);
-        atomicAdd(sgw + 2 * wn + jw + 1, fw * g_om1 * facv.z);
-        atomicAdd(sgw + 3 * wn + jw + 1, fw * g_om2 * facv.w);
+    const float g[4] = {g_u1 * facv.x, g_u2 * facv.y, g_om1 * facv.z, g_om2 * facv.w};
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        ws.a0[q] = fmaf(a0, g[q], ws.a0[q]);
+        if (fw != 0.f) ws.a1[q] = fmaf(fw, g[q], ws.a1[q]);
     }
     gl[0] = fmaf(g_u1, u1w, gl[0]);
     gl[1] = fmaf(g_u2, u2w, gl[1]);
@@ -432,7 +500,7 @@ __device__ __forceinline__ void flush_stage(const DoseArgs& a, const int2* st, i
 template <int MODE, int NF, bool MERGED, int LAT, int PREC = 0>
 __device__ __forceinline__ void process_unit(const DoseArgs& a, const int32_t vi, const int64_t e0, const int b,
                                              const float4* __restrict__ sW, int2* sst, float4* srow,
-                                             const int lane, uint32_t* stc = nullptr)
+                                             const int lane, uint32_t* stc = nullptr, const int split = 0)
 {
     // the tensor-core form of 64 fluence vectors; its pair values in FP32
     // exponentials like the plain form
@@ -451,6 +519,7 @@ __device__ __forceinline__ void process_unit(const DoseArgs& a, const int32_t vi
     const BeamDev& bm = P.beams[b];
     float4 facv = make_float4(0.f, 0.f, 0.f, 0.f);
     float gl[4] = {0.f, 0.f, 0.f, 0.f}, gc[2] = {0.f, 0.f};
+    WaterSums ws{-1, {0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};
     const float wgt = MODE == kGrad && ln.valid ? __ldg(a.wv + v) : 0.f;   // voxel weight of the backward pass
     if (MODE != kCount) {
         const float4 fac = __ldg(P.fac + v);   // f_u1(rho), f_u2(rho_hat), f_w1(rho_hat), f_w2(rho_hat)
@@ -503,7 +572,8 @@ __device__ __forceinline__ void process_unit(const DoseArgs& a, const int32_t vi
     }
     const int wnlo = __reduce_min_sync(0xffffffffu, nlo);
     const int wnhi = __reduce_max_sync(0xffffffffu, nhi);
-    for (int n = wnlo; n <= wnhi; ++n) {
+    // (the backward pass takes every kGradSplit-th row of a work item's window)
+    for (int n = wnlo + (MODE == kGrad ? split : 0); n <= wnhi; n += MODE == kGrad ? kGradSplit : 1) {
         const float dc_ = cc - (-hfy + (n + 0.5f) * P.by);
         const float h2 = rw * rw - dc_ * dc_;
         int mlo = INT_MAX, mhi = INT_MIN;
@@ -573,7 +643,7 @@ __device__ __forceinline__ void process_unit(const DoseArgs& a, const int32_t vi
             if (MODE == kGrad) {
                 if (pt.in && wgt != 0.f)
                     pair_grad(P, facv, i, sad, sW, pt, wgt * rq[2].w,
-                              reinterpret_cast<float*>(sst), gl, gc);
+                              reinterpret_cast<float*>(sst), ws, gl, gc);
                 continue;
             }
             if (TC) {
@@ -626,23 +696,32 @@ __device__ __forceinline__ void process_unit(const DoseArgs& a, const int32_t vi
         }
     }
     if (MODE == kGrad) {
-        if (ln.valid && wgt != 0.f) {
-            // the per-voxel derivatives go to the bins of rho (f_u1) and rho_hat (the others)
-            float* sgd = reinterpret_cast<float*>(sst) + 4 * P.w_n;
-            int j;
-            float w;
-            dens_bins(P, __ldg(P.rho + v), j, w);
-            atomicAdd(sgd + j, (1.f - w) * gl[0]);
-            atomicAdd(sgd + j + 1, w * gl[0]);
-            dens_bins(P, __ldg(P.rhos + v), j, w);
+        float* sgw = reinterpret_cast<float*>(sst);
+        float* sgd = sgw + 4 * P.w_n;
+        const float vw[8] = {ws.a0[0], ws.a0[1], ws.a0[2], ws.a0[3], ws.a1[0], ws.a1[1], ws.a1[2], ws.a1[3]};
+        add_by_key(ws.j, ws.j >= 0, vw, lane, [&](int j, int q) -> float* {
+            j += q >> 2;
+            return j < P.w_n ? sgw + (q & 3) * P.w_n + j : nullptr;
+        });
 #pragma unroll
-            for (int q = 1; q < 4; ++q) {
-                atomicAdd(sgd + q * P.f_n + j, (1.f - w) * gl[q]);
-                atomicAdd(sgd + q * P.f_n + j + 1, w * gl[q]);
-            }
-            atomicAdd(sgd + 4 * P.f_n, gc[0]);
-            atomicAdd(sgd + 4 * P.f_n + 1, gc[1]);
+        for (int q = 0; q < 2; ++q) {
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) gc[q] += __shfl_xor_sync(0xffffffffu, gc[q], o);
+            if (lane == 0) atomicAdd(sgd + 4 * P.f_n + q, gc[q]);
         }
+        // the per-voxel derivatives go to the bins of rho (f_u1) and rho_hat (the others)
+        const bool on = ln.valid && wgt != 0.f;
+        int j0 = 0, j1 = 0;
+        float w0 = 0.f, w1 = 0.f;
+        if (on) {
+            dens_bins(P, __ldg(P.rho + v), j0, w0);
+            dens_bins(P, __ldg(P.rhos + v), j1, w1);
+        }
+        const float vd[8] = {(1.f - w0) * gl[0], w0 * gl[0], (1.f - w1) * gl[1], w1 * gl[1],
+                             (1.f - w1) * gl[2], w1 * gl[2], (1.f - w1) * gl[3], w1 * gl[3]};
+        add_by_key(j0 * P.f_n + j1, on, vd, lane, [&](int key, int q) -> float* {
+            return q < 2 ? sgd + key / P.f_n + q : sgd + (q >> 1) * P.f_n + key % P.f_n + (q & 1);
+        });
     } else if (TC) {
         // accumulator (tile t, vectors 8u .. 8u + 7, element 2h + e) is row
         // 16t + 8h + g (that lane's voxel), vector 8u + 2 t4 + e
@@ -721,18 +800,19 @@ __global__ void __launch_bounds__(kThreads, MINB) k_pairs(const DoseArgs a)
     for (int q = threadIdx.x; q <= P.n_beams; q += blockDim.x) s_base[q] = a.base[q];
     __syncthreads();
     const int total = a.work[0];
+    constexpr int kItems = MODE == kGrad ? kGradSplit : 1;   // work items per unit
 
     for (;;) {
         int w = 0;
         if (lane == 0) w = atomicAdd(a.work + 1, 1);
         w = __shfl_sync(0xffffffffu, w, 0);
-        if (w >= total) break;
-        const int64_t e0 = (int64_t)DC_GUARD(P, w, (s_base[P.n_beams] + 31) / 32, 4) * 32;
+        if (w / kItems >= total) break;
+        const int64_t e0 = (int64_t)DC_GUARD(P, w / kItems, (s_base[P.n_beams] + 31) / 32, 4) * 32;
         int b = 0;
         while (b + 1 < P.n_beams && s_base[b + 1] <= e0) ++b;
         const int32_t vi = __ldg(a.items + e0 + lane);
         process_unit<MODE, NF, MERGED, LAT, PREC>(a, vi, e0, b, sW, sst, s_row[warp], lane,
-                                                  TC ? s_tc[TC ? warp : 0] : nullptr);
+                                                  TC ? s_tc[TC ? warp : 0] : nullptr, w % kItems);
     }
     if (MODE == kGrad) {
         __syncthreads();
