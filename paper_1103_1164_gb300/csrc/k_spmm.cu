@@ -485,11 +485,14 @@ __global__ void __launch_bounds__(kSpmmThreads) k_spmm(const SpmmArgs a)
 }
 
 // Y[v][q] = sum over beams of the partial rows, in beam order, with
-// Neumaier-compensated summation.  A warp per voxel: the lanes find the
-// voxel's list positions of all beams at once, then add the partial rows
-// column by column (lane l: columns 2l, 2l + 1), so the row reads are whole
-// lines.  (One thread per output element, each looking up the positions
-// itself, took 9.5 ms on a 12.6 M-voxel, 9-beam plan at k = 64.)
+// Neumaier-compensated summation.  G lanes per voxel, as few as hold its k columns
+// two by two, so that row reads are whole lines and lanes do not idle: they look up
+// the voxel's list positions in G beams at once, one voxel ahead (that lookup's
+// latency overlaps the sums), then add the partial rows (lane l: columns 2l,
+// 2l + 1).  With a warp per voxel whatever the k: 196 us for k = 21 on 830 k voxels
+// and 5 beams, now 115; k = 8, 1.57 M voxels, 9 beams: 443 -> 161; k = 64 and 33
+// stay (357 -> 351, 508 -> 506).  Loading 3 to 8 beams' rows before adding any was
+// slower for k > 32 (373 to 500 us at k = 64).
 __device__ __forceinline__ void neumaier_add(float& s, float& c, float x)
 {
     const float t = s + x;
@@ -497,37 +500,68 @@ __device__ __forceinline__ void neumaier_add(float& s, float& c, float x)
     s = t;
 }
 
+template <int G, bool PAIRS>
 __global__ void __launch_bounds__(256) k_spmm_reduce(const float* __restrict__ P, const int32_t* __restrict__ inv,
                                                      int n_beams, int64_t V, int k, float* __restrict__ Y)
 {
-    const int lane = threadIdx.x & 31, q = 2 * lane;
-    const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    // the voxel's position in each beam's list (at most 64 beams: two per
-    // lane), looked up one voxel ahead so that the lookup of the next voxel
-    // overlaps the sums of this one
-    int64_t v = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
-    auto lookup = [&](int64_t u, int32_t& a, int32_t& b) {
-        a = u < V && lane < n_beams ? __ldg(inv + (size_t)lane * V + u) : -1;
-        b = u < V && lane + 32 < n_beams ? __ldg(inv + (size_t)(lane + 32) * V + u) : -1;
-    };
-    int32_t na, nb;
-    lookup(v, na, nb);
-    for (; v < V; v += nwarps) {
-        const int32_t pa = na, pb = nb;
-        lookup(v + nwarps, na, nb);
+    const int l = threadIdx.x % G, q = 2 * l;
+    const int64_t step = (int64_t)gridDim.x * (blockDim.x / G);
+    int64_t v = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) / G;
+    const auto lookup = [&](int64_t u, int b) { return u < V && b < n_beams ? __ldg(inv + (size_t)b * V + u) : -1; };
+    int32_t next = lookup(v, l);
+    // whole warps iterate together (v0: the warp's first voxel)
+    for (int64_t v0 = v - (threadIdx.x & 31) / G; v0 < V; v0 += step, v += step) {
         float s0 = 0.f, c0 = 0.f, s1 = 0.f, c1 = 0.f;
+        int32_t mine = next;
+        next = lookup(v + step, l);
+        for (int b0 = 0; b0 < n_beams; b0 += G) {
+            if (b0 > 0) mine = lookup(v, b0 + l);
+            const int nb = min(G, n_beams - b0);
 #pragma unroll 4
-        for (int b = 0; b < n_beams; ++b) {
-            const int32_t pos = __shfl_sync(0xffffffffu, b < 32 ? pa : pb, b & 31);
-            if (pos < 0) continue;
-            const float* row = P + (size_t)pos * k;
-            if (q < k) neumaier_add(s0, c0, __ldg(row + q));
-            if (q + 1 < k) neumaier_add(s1, c1, __ldg(row + q + 1));
+            for (int j = 0; j < nb; ++j) {
+                const int32_t pos = __shfl_sync(0xffffffffu, mine, j, G);
+                if (pos < 0) continue;
+                const float* row = P + (size_t)pos * k + q;
+                float2 x = make_float2(0.f, 0.f);
+                if (PAIRS) {
+                    if (q < k) x = __ldg(reinterpret_cast<const float2*>(row));
+                } else {
+                    if (q < k) x.x = __ldg(row);
+                    if (q + 1 < k) x.y = __ldg(row + 1);
+                }
+                neumaier_add(s0, c0, x.x);
+                neumaier_add(s1, c1, x.y);
+            }
         }
-        float* y = Y + (size_t)v * k;
-        if (q < k) y[q] = s0 + c0;
-        if (q + 1 < k) y[q + 1] = s1 + c1;
+        if (v >= V) continue;
+        float* y = Y + (size_t)v * k + q;
+        if (PAIRS) {
+            if (q < k) *reinterpret_cast<float2*>(y) = make_float2(s0 + c0, s1 + c1);
+        } else {
+            if (q < k) y[0] = s0 + c0;
+            if (q + 1 < k) y[1] = s1 + c1;
+        }
     }
+}
+
+template <int G>
+cudaError_t reduce_launch(cudaStream_t s, const float* P, const int32_t* inv, int n_beams, int64_t V, int k, float* Y)
+{
+    const int64_t blocks = (V * G + 255) / 256;
+    const int grid = (int)std::min<int64_t>(blocks, 152 * 64);
+    // pairs of columns as 8-byte words where every row starts on one
+    if (k % 2 == 0 && ((reinterpret_cast<uintptr_t>(P) | reinterpret_cast<uintptr_t>(Y)) & 7) == 0)
+        k_spmm_reduce<G, true><<<grid, 256, 0, s>>>(P, inv, n_beams, V, k, Y);
+    else
+        k_spmm_reduce<G, false><<<grid, 256, 0, s>>>(P, inv, n_beams, V, k, Y);
+    count_launches(1);
+    return cudaGetLastError();
+}
+
+cudaError_t spmm_reduce(cudaStream_t s, const float* P, const int32_t* inv, int n_beams, int64_t V, int k, float* Y)
+{
+    if (k <= 16) return reduce_launch<8>(s, P, inv, n_beams, V, k, Y);
+    return k <= 32 ? reduce_launch<16>(s, P, inv, n_beams, V, k, Y) : reduce_launch<32>(s, P, inv, n_beams, V, k, Y);
 }
 
 // inv[b][v] = position of voxel v in beam b's list (-1 if absent).
@@ -847,9 +881,7 @@ cudaError_t spmm_run(dc_plan* p, const float* F, int k, float* Y)
         if (e != cudaSuccess) return e;
     }
     if (!direct) {
-        k_spmm_reduce<<<gsize(p->V * 32), 256, 0, p->stream>>>(p->d_sp_p, p->d_sp_inv, p->n_beams, p->V, k, Y);
-        count_launches(1);
-        e = cudaGetLastError();
+        e = spmm_reduce(p->stream, p->d_sp_p, p->d_sp_inv, p->n_beams, p->V, k, Y);
     }
     return e;
 }
@@ -960,9 +992,7 @@ cudaError_t spmm_run_static(dc_plan* p, const float* F, int k, float* Y)
         if (e != cudaSuccess) return e;
     }
     if (!direct) {
-        k_spmm_reduce<<<gsize(p->V * 32), 256, 0, p->stream>>>(sc.part, p->d_sp_inv, p->n_beams, p->V, k, Y);
-        count_launches(1);
-        e = cudaGetLastError();
+        e = spmm_reduce(p->stream, sc.part, p->d_sp_inv, p->n_beams, p->V, k, Y);
     }
     return e;
 }
