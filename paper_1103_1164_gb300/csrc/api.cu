@@ -423,7 +423,7 @@ static dc_status create_impl(dc_plan* p, const float* ct, uint32_t flags)
     DC_CUDA(dalloc(&p->d_bstart, nb + 1));
     DC_CUDA(dalloc(&p->d_bscan, (nb * (size_t)p->cells_cap + 4095) / 4096 + 2));
     DC_CUDA(dalloc(&p->d_base, nb + 1));
-    DC_CUDA(dalloc(&p->d_work, 2));
+    DC_CUDA(dalloc(&p->d_work, 4));
     DC_CUDA(dalloc(&p->d_items, nb * (V + 32)));
     DC_CUDA(dalloc(&p->d_part, nb * V));
     p->part_cap = nb * V;

@@ -74,7 +74,7 @@ struct dc_plan {
     int32_t* d_bstart = nullptr;     // [n_beams + 1] start of each beam's cells in the device-wide cell scan
     int32_t* d_bscan = nullptr;      // chunk sums of that scan
     int64_t* d_base = nullptr;       // [n_beams + 1] start of each beam's list (whole warps)
-    int32_t* d_work = nullptr;       // [0] warp work units, [1] work counter
+    int32_t* d_work = nullptr;       // warp work units and counter; the same for the single-fluence dose
     int32_t* d_items = nullptr;      // [n_beams][V + 32]
     float* d_part = nullptr;         // per-beam partial dose [n_beams][V][vectors of a pass]
     size_t part_cap = 0;

@@ -258,7 +258,8 @@ __global__ void k_bin_bases(int n_beams, const int32_t* __restrict__ bstart, int
         s += ((int64_t)nb + 31) / 32 * 32;
     }
     base[n_beams] = s;
-    work[0] = (int32_t)(s / 32);
+    work[0] = work[2] = (int32_t)(s / 32);
+    work[3] = 0;   // the dose's counter (k_sum_beams)
 }
 
 // Pass 4: scatter voxel indices into their beam's list, grouped by cell;

@@ -1767,8 +1767,10 @@ __global__ void __launch_bounds__(256) k_sum_batch(const DoseArgs* __restrict__ 
 // (`cell` >= 0 says which: the partials of the others are neither written nor
 // cleared).
 __global__ void __launch_bounds__(256) k_sum_beams(const float* __restrict__ part, const int32_t* __restrict__ cell,
-                                                   int n_beams, int64_t V, float* __restrict__ dose)
+                                                   int n_beams, int64_t V, float* __restrict__ dose,
+                                                   int32_t* dose_counter)
 {
+    if (blockIdx.x == 0 && threadIdx.x == 0) *dose_counter = 0;
     for (int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; v < V; v += (int64_t)gridDim.x * blockDim.x) {
         float s = 0.f;
 #pragma unroll 4
@@ -1903,10 +1905,10 @@ int grid_for(int64_t n)
     return (int)(g > 152 * 32 ? 152 * 32 : (g < 1 ? 1 : g));
 }
 
-// Persistent launch of a kernel that takes its units from the plan's counter:
-// as many CTAs as fit on the device at once.
+// Persistent launch of a kernel that takes its units from one of the plan's
+// counters, which is zero: as many CTAs as fit on the device at once.
 template <typename K, typename... Args>
-cudaError_t launch_units(const dc_plan* p, K kern, size_t sm, const Args&... args)
+cudaError_t launch_zeroed(const dc_plan* p, K kern, size_t sm, const Args&... args)
 {
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     if (e != cudaSuccess) return e;
@@ -1915,11 +1917,17 @@ cudaError_t launch_units(const dc_plan* p, K kern, size_t sm, const Args&... arg
     if (e != cudaSuccess) return e;
     e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, p->device);
     if (e != cudaSuccess) return e;
-    e = cudaMemsetAsync(p->d_work + 1, 0, sizeof(int32_t), p->stream);
-    if (e != cudaSuccess) return e;
     kern<<<sms * (per_sm > 0 ? per_sm : 1), kThreads, sm, p->stream>>>(args...);
     count_launches(1);
     return cudaGetLastError();
+}
+
+// The same with the counter of d_work[1], which is cleared here.
+template <typename K, typename... Args>
+cudaError_t launch_units(const dc_plan* p, K kern, size_t sm, const Args&... args)
+{
+    const cudaError_t e = cudaMemsetAsync(p->d_work + 1, 0, sizeof(int32_t), p->stream);
+    return e != cudaSuccess ? e : launch_zeroed(p, kern, sm, args...);
 }
 
 template <int MODE, int NF, bool MERGED, int LAT, int PREC = 0>
@@ -1932,7 +1940,8 @@ cudaError_t run_variant(const dc_plan* p, const DoseArgs& a)
         if (e != cudaSuccess) return e;
         // no more units than warps with 4 CTAs per SM
         if ((int64_t)p->n_beams * ((p->V + 31) / 32) <= (int64_t)sms * 4 * kWarps)
-            return launch_units(p, k_pairs<MODE, NF, MERGED, LAT, PREC, 4>, sm, a);
+            return launch_zeroed(p, k_pairs<MODE, NF, MERGED, LAT, PREC, 4>, sm, a);
+        return launch_zeroed(p, k_pairs<MODE, NF, MERGED, LAT, PREC>, sm, a);
     }
     return launch_units(p, k_pairs<MODE, NF, MERGED, LAT, PREC>, sm, a);
 }
@@ -2101,9 +2110,13 @@ cudaError_t launch_dose(const dc_plan* p, const float* fluence, int nf, int ldf,
         a.count_out = p->d_bcount;
     }
     if (p->part_cap < (size_t)p->n_beams * p->V) return cudaErrorInvalidValue;
+    // the dose has a counter of its own, zeroed by the binning and by k_sum_beams
+    // after each pass: no clearing of 2 us before the smallest plans' 32
+    a.work = p->d_work + 2;
     const cudaError_t e = run<kDose, 1>(p, a);
     if (e != cudaSuccess) return e;
-    k_sum_beams<<<grid_for(p->V), 256, 0, p->stream>>>(p->d_part, p->d_cellof, p->n_beams, p->V, dose);
+    k_sum_beams<<<grid_for(p->V), 256, 0, p->stream>>>(p->d_part, p->d_cellof, p->n_beams, p->V, dose,
+                                                        p->d_work + 3);
     count_launches(1);
     return cudaGetLastError();
 }
@@ -2155,7 +2168,8 @@ cudaError_t launch_fill(const dc_plan* p, const int64_t* rowptr, int32_t* cols, 
     a.part = p->d_part;
     cudaError_t e = run<kFill, 1>(p, a);
     if (e != cudaSuccess) return e;
-    k_sum_beams<<<grid_for(p->V), 256, 0, p->stream>>>(p->d_part, p->d_cellof, p->n_beams, p->V, dose);
+    k_sum_beams<<<grid_for(p->V), 256, 0, p->stream>>>(p->d_part, p->d_cellof, p->n_beams, p->V, dose,
+                                                        p->d_work + 3);
     count_launches(1);
     return cudaGetLastError();
 }
