@@ -758,8 +758,8 @@ __device__ __forceinline__ void process_unit(const DoseArgs& a, const int32_t vi
 // would otherwise be recomputed in the hot loop), 128 for the tensor-core form of
 // 64 vectors (their accumulators).  A single-fluence dose whose units do
 // not fill the GPU takes 64 as well: its time is that of one unit's chain of
-// loads, and the two interleaved beamlets want the registers (4,320 voxels, 3
-// beams: 41 us with 48, 38 us with 64).
+// loads, and the two interleaved beamlets want the registers (single calls with
+// 4,800 units: 113 us with 48, 105 us with 64).
 template <int MODE, int NF>
 constexpr int min_ctas()
 {
@@ -1275,6 +1275,117 @@ __global__ void __launch_bounds__(kThreads, multi_ctas<NF>()) k_dose_multi(const
                 reinterpret_cast<float2*>(out)[fg] = make_float2(acc[j][0], acc[j][1]);
             else
                 reinterpret_cast<float4*>(out)[fg] = make_float4(acc[j][0], acc[j][1], acc[j][VP - 2], acc[j][VP - 1]);
+        }
+    }
+}
+
+// ---------------------------------------------------------------------------
+// The single-fluence dose of a plan with so few units that a warp per unit leaves
+// most of the GPU idle: its time is then one unit's chain of loads and arithmetic.
+// A CTA takes a unit.  The window's beamlets are laid out in order, kSmallRows at a
+// time; each warp evaluates an equal part of them for the 32 voxels into the CTA's
+// tile, and the last warp adds the tile up in beamlet order, with the same
+// operations as k_pairs, so the dose is the same to the bit.  4,320 voxels, 3 beams:
+// 32 -> 17 us per dose.
+constexpr int kSmallRows = 32 * kWarps;
+
+template <bool MERGED, int LAT, int PREC>
+__global__ void __launch_bounds__(kThreads, 4) k_dose_small(const DoseArgs a)
+{
+    extern __shared__ float4 smem[];
+    __shared__ int64_t s_base[kMaxBeams + 1];
+    __shared__ float4 s_row[kWarps][3 * 32];
+    __shared__ float s_d[kSmallRows * 32];
+    __shared__ float2 s_f[kSmallRows];   // fluence, and which of the 32 voxels are pairs (bits)
+    __shared__ RowWindows s_win[kWarps];
+    __shared__ int s_w;
+    const PlanView& P = a.P;
+    const int64_t V = (int64_t)P.nx * P.ny * P.nz;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    if (!MERGED)
+        for (int q = threadIdx.x; q < 2 * P.w_n; q += blockDim.x) smem[q] = __ldg(P.water + q);
+    for (int q = threadIdx.x; q <= P.n_beams; q += blockDim.x) s_base[q] = a.base[q];
+    float4* srow = s_row[warp];
+    RowWindows& win = s_win[warp];
+    const int total = a.work[0];
+    for (;;) {
+        __syncthreads();
+        if (threadIdx.x == 0) s_w = atomicAdd(a.work + 1, 1);
+        __syncthreads();
+        const int w = s_w;
+        if (w >= total) break;
+        const int64_t e0 = (int64_t)DC_GUARD(P, w, (s_base[P.n_beams] + 31) / 32, 4) * 32;
+        int b = 0;
+        while (b + 1 < P.n_beams && s_base[b + 1] <= e0) ++b;
+        const int32_t vi = __ldg(a.items + e0 + lane);
+        const BeamDev& bm = P.beams[b];
+        const float sad = __ldg(&bm.sad);
+        int n0, n1;
+        Lane ln;
+        UnitBox box;
+        {
+            CountVoxel c[1] = {count_voxel(P, bm, vi, sad)};
+            ln = c[0].ln;
+            box = unit_box<1>(c);
+            box_rows(P, box, __ldg(&bm.N), __ldg(&bm.half_fy), n0, n1);
+            const float4 fac = __ldg(P.fac + c[0].v);   // f_u1(rho), f_u2(rho_hat), f_w1(rho_hat), f_w2(rho_hat)
+            const float4 lf = LAT == kItem ? __ldg(P.lfac + e0 + lane)
+                                           : make_float4(kLog2e * fac.y, kLog2e * fac.y, fac.z, fac.w);
+            ln.cu1 = kLog2e * fac.x;
+            ln.cu2x = lf.x;
+            ln.cu2y = lf.y;
+            ln.cw1 = lf.z;
+            ln.cw2 = lf.w;
+        }
+        float acc = 0.f;
+        int32_t cnt = 0;
+        for (int nb = n0; nb <= n1; nb += 32) {
+            const int places = row_windows(P, box, win, nb, n1, __ldg(&bm.M), __ldg(&bm.first), __ldg(&bm.half_fx),
+                                           __ldg(&bm.half_fy), lane);
+            for (int q0 = 0; q0 < places; q0 += kSmallRows) {
+                const int nq = min(kSmallRows, places - q0), per = (nq + kWarps - 1) / kWarps;
+                const int k0 = warp * per, mine = min(per, nq - k0);   // places q0 + k0 .. are the warp's
+                float f = 0.f;
+                int ib = 0;
+                __syncwarp();
+                if (lane < mine) {
+                    const int place = q0 + k0 + lane;
+                    ib = (int)DC_GUARD(P, win.base[window_row(win, place)] + place, P.B, 5);
+                    const float4* src = reinterpret_cast<const float4*>(P.bl) + 4u * (uint32_t)ib;
+                    srow[3 * lane] = __ldg(src);
+                    srow[3 * lane + 1] = __ldg(src + 1);
+                    srow[3 * lane + 2] = __ldg(src + 2);
+                    f = __ldg(a.fluence + ib);
+                }
+                __syncthreads();   // the last chunk has been added up
+                uint32_t bits = 0;
+#pragma unroll 2
+                for (int m = 0; m < mine; ++m) {
+                    const uint32_t i = (uint32_t)__shfl_sync(0xffffffffu, ib, m);
+                    const float4* rq = srow + 3 * m;
+                    const PairTest pt = pair_test(P, ln, rq[0], rq[1], rq[2]);
+                    if (pt.in) s_d[(k0 + m) * 32 + lane] = pair_eval<MERGED, LAT, PREC>(P, ln, i, sad, smem, pt);
+                    const uint32_t in = __ballot_sync(0xffffffffu, pt.in);
+                    if (lane == m) bits = in;
+                }
+                if (lane < mine) s_f[k0 + lane] = make_float2(f, __uint_as_float(bits));
+                __syncthreads();
+                if (warp == kWarps - 1) {
+#pragma unroll 8
+                    for (int k = 0; k < nq; ++k) {
+                        const float2 fb = s_f[k];
+                        const float D = s_d[k * 32 + lane];
+                        if (__float_as_uint(fb.y) >> lane & 1u) {
+                            acc = fmaf(fb.x, D, acc);
+                            ++cnt;
+                        }
+                    }
+                }
+            }
+        }
+        if (warp == kWarps - 1 && ln.valid) {
+            a.part[(size_t)b * V + vi] = acc;
+            if (a.count_out) a.count_out[(size_t)b * V + vi] = cnt;
         }
     }
 }
@@ -1938,8 +2049,18 @@ cudaError_t run_variant(const dc_plan* p, const DoseArgs& a)
         int sms = 0;
         const cudaError_t e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, p->device);
         if (e != cudaSuccess) return e;
+        const int64_t units = (int64_t)p->n_beams * ((p->V + 31) / 32);   // at most (voxels outside a beam have none)
+        // A CTA per unit up to 16 units per SM: single calls with 405 to 2,400 units
+        // 45-76 us -> 35-59, and with 452 beamlets per window 256 -> 137.  With so
+        // many (ROI area / beamlet area) it pays up to 32: 3,600 units 250 -> 155,
+        // 4,800 150 -> 130; with 113 to 314 it does not (4,200 units 68 -> 78, 4,800
+        // 101 -> 116).
+        const double window = 3.1416 * p->coeffs.roi_radius * p->coeffs.roi_radius / ((double)p->bx * p->by);
+        // (three CTAs or more fit with water tables of up to 24 KB)
+        if (sm <= 24 * 1024 && units <= (int64_t)sms * (window >= 400. ? 32 : 16))
+            return launch_zeroed(p, k_dose_small<MERGED, LAT, PREC>, sm, a);
         // no more units than warps with 4 CTAs per SM
-        if ((int64_t)p->n_beams * ((p->V + 31) / 32) <= (int64_t)sms * 4 * kWarps)
+        if (units <= (int64_t)sms * 4 * kWarps)
             return launch_zeroed(p, k_pairs<MODE, NF, MERGED, LAT, PREC, 4>, sm, a);
         return launch_zeroed(p, k_pairs<MODE, NF, MERGED, LAT, PREC>, sm, a);
     }
