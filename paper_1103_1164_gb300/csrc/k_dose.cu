@@ -39,7 +39,7 @@ constexpr int kRingLd = kRing + 1;
 // 32 fluence vectors, whose staging does
 constexpr int row_max(int mode, int nf = 1) { return mode == 2 || nf > 32 ? 16 : 32; }
 
-enum Mode { kDose = 0, kCount = 1, kFill = 2, kGrad = 3 };
+enum Mode { kDose = 0, kFill = 2, kGrad = 3 };
 // work items per unit of the backward pass, whose phantoms have few units (a 60^3
 // grid: 6,750 for 4,864 warps, so whole units ran in two rounds).  A single call on
 // that grid: 385 us with 1 item, 254 with 2, 200 with 4, 220 with 8; 30^3: 225, 156,
@@ -521,21 +521,19 @@ __device__ __forceinline__ void process_unit(const DoseArgs& a, const int32_t vi
     float gl[4] = {0.f, 0.f, 0.f, 0.f}, gc[2] = {0.f, 0.f};
     WaterSums ws{-1, {0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};
     const float wgt = MODE == kGrad && ln.valid ? __ldg(a.wv + v) : 0.f;   // voxel weight of the backward pass
-    if (MODE != kCount) {
-        const float4 fac = __ldg(P.fac + v);   // f_u1(rho), f_u2(rho_hat), f_w1(rho_hat), f_w2(rho_hat)
-        facv = fac;
-        ln.cu1 = kLog2e * fac.x;
-        ln.cu2x = ln.cu2y = kLog2e * fac.y;
-        ln.cw1 = fac.z;
-        ln.cw2 = fac.w;
-        if (LAT == kItem) {
-            // (log2(e) f_u2 along x, along y, f_w1, f_w2) of this (voxel, beam)
-            const float4 lf = __ldg(P.lfac + e0 + lane);   // e0 + lane: guarded with the list entry (code 4)
-            ln.cu2x = lf.x;
-            ln.cu2y = lf.y;
-            ln.cw1 = lf.z;
-            ln.cw2 = lf.w;
-        }
+    const float4 fac = __ldg(P.fac + v);   // f_u1(rho), f_u2(rho_hat), f_w1(rho_hat), f_w2(rho_hat)
+    facv = fac;
+    ln.cu1 = kLog2e * fac.x;
+    ln.cu2x = ln.cu2y = kLog2e * fac.y;
+    ln.cw1 = fac.z;
+    ln.cw2 = fac.w;
+    if (LAT == kItem) {
+        // (log2(e) f_u2 along x, along y, f_w1, f_w2) of this (voxel, beam)
+        const float4 lf = __ldg(P.lfac + e0 + lane);   // e0 + lane: guarded with the list entry (code 4)
+        ln.cu2x = lf.x;
+        ln.cu2y = lf.y;
+        ln.cw1 = lf.z;
+        ln.cw2 = lf.w;
     }
     float acc[NF > 0 ? NF : 1];
 #pragma unroll
@@ -599,7 +597,7 @@ __device__ __forceinline__ void process_unit(const DoseArgs& a, const int32_t vi
             float4 q2 = __ldg(src + 2);
             // one fluence vector: the staged record carries f_i in place of the
             // theta weight (which only the table set-up uses)
-            if (MODE != kCount && NF == 1) q2.w = __ldg(a.fluence + ib);
+            if (NF == 1) q2.w = __ldg(a.fluence + ib);
             srow[3 * lane + 2] = q2;
         }
         if (TC) {
@@ -636,10 +634,6 @@ __device__ __forceinline__ void process_unit(const DoseArgs& a, const int32_t vi
             const uint32_t i = row + (uint32_t)m;
             const float4* rq = srow + 3 * (m - m0);
             const PairTest pt = pair_test(P, ln, rq[0], rq[1], rq[2]);
-            if (MODE == kCount) {
-                cnt += pt.in ? 1 : 0;
-                continue;
-            }
             if (MODE == kGrad) {
                 if (pt.in && wgt != 0.f)
                     pair_grad(P, facv, i, sad, sW, pt, wgt * rq[2].w,
@@ -741,12 +735,8 @@ __device__ __forceinline__ void process_unit(const DoseArgs& a, const int32_t vi
         flush_stage(a, sst, lane, cnt, pos, pend, mis, true);
         if (NF == 1 && ln.valid) a.part[(size_t)b * V + v] = acc[0];
     } else if (ln.valid) {
-        if (MODE == kDose) {
-            a.part[(size_t)b * V + v] = acc[0];
-            if (a.count_out) a.count_out[(size_t)b * V + v] = cnt;
-        } else {
-            a.bcount[(size_t)b * V + v] = cnt;
-        }
+        a.part[(size_t)b * V + v] = acc[0];
+        if (a.count_out) a.count_out[(size_t)b * V + v] = cnt;
     }
 }
 
@@ -754,7 +744,7 @@ __device__ __forceinline__ void process_unit(const DoseArgs& a, const int32_t vi
 // of one or two neighbouring beam's-eye-view cells; -1 entries are padding).
 // Persistent CTAs take units from a global counter.
 // Register budgets: 48 per thread for the single-fluence dose (5 CTAs per
-// SM), 64 for the pair count and the CSR fill (4 CTAs; the fill's extra state
+// SM), 64 for the CSR fill and the backward pass (4 CTAs; the fill's extra state
 // would otherwise be recomputed in the hot loop), 128 for the tensor-core form of
 // 64 vectors (their accumulators).  A single-fluence dose whose units do
 // not fill the GPU takes 64 as well: its time is that of one unit's chain of
@@ -763,7 +753,7 @@ __device__ __forceinline__ void process_unit(const DoseArgs& a, const int32_t vi
 template <int MODE, int NF>
 constexpr int min_ctas()
 {
-    return MODE == kCount || MODE == kFill || MODE == kGrad ? 4 : (NF == 1 ? 5 : 2);
+    return MODE == kFill || MODE == kGrad ? 4 : (NF == 1 ? 5 : 2);
 }
 
 template <int MODE, int NF, bool MERGED, int LAT, int PREC, int MINB = min_ctas<MODE, NF>()>
@@ -795,7 +785,7 @@ __global__ void __launch_bounds__(kThreads, MINB) k_pairs(const DoseArgs a)
         for (int q = threadIdx.x & 31; q < kTcOffF; q += 32) s_tc[threadIdx.x >> 5][q] = 0u;
     }
     // the water tables are read from shared memory unless merged into the depth tables
-    if (MODE != kCount && !MERGED)
+    if (!MERGED)
         for (int q = threadIdx.x; q < 2 * P.w_n; q += blockDim.x) sW[q] = __ldg(P.water + q);
     for (int q = threadIdx.x; q <= P.n_beams; q += blockDim.x) s_base[q] = a.base[q];
     __syncthreads();
@@ -2024,7 +2014,6 @@ DoseArgs make_args(const dc_plan* p)
 
 size_t smem_bytes(const dc_plan* p, int mode)
 {
-    if (mode == kCount) return 0;
     if (mode == kGrad)   // water tables + gradient bins (always the general tables)
         return 2 * sizeof(float4) * p->coeffs.w_n + sizeof(float) * (4 * (size_t)p->coeffs.w_n + 4 * p->coeffs.f_n + 2);
     size_t s = p->merged ? 0 : 2 * sizeof(float4) * p->coeffs.w_n;
@@ -2133,7 +2122,6 @@ cudaError_t run_multi(const dc_plan* p, const DoseArgs& a, float* dose, int64_t 
 template <int MODE, int NF>
 cudaError_t run(const dc_plan* p, const DoseArgs& a)
 {
-    if (MODE == kCount) return run_variant<kCount, 1, false, kIso>(p, a);
     // per-item factors exist for the axis and network forms with the density correction on
     const bool item = p->coeffs.density_correction && p->lateral_mode != DC_LATERAL_ISO;
     if (MODE == kDose && NF == 1 && p->precision == DC_PRECISION_BF16) {
