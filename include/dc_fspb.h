@@ -186,13 +186,14 @@ dc_status dc_fspb_dose(dc_plan* plan, const float* fluence, float* dose, uint32_
 /*
  * Eq. (1) for k fluence vectors at once: dose[q][v] = sum_i fluence[q][i] D_i(r_v),
  * each D_i(r_v) evaluated once and applied to all k vectors (1 <= k <= 64):
- * one pass of 16, 32 or 64 vectors (the smallest that holds k), with the
- * beamlets' fluences staged beside their records.  For k > 1 each vector's
+ * one pass of 16, 32 or 64 vectors (the smallest that holds k), a
+ * register-tiled product of shared pair values and fluences.  For k > 1 each vector's
  * dose is the same, bit for bit, whatever k it is computed with.
  *   fluence [k][B]; dose [k][V].
  * Scratch, kept by the plan: per-beam partial doses, n_beams * width * V
  * floats (width 16, 32 or 64; 64 in the tensor-core form of
- * DC_PRECISION_BF16), and in that form the fluences packed as B * 64 BF16.
+ * DC_PRECISION_BF16), and the fluences packed as B * width floats (B * 64 BF16
+ * in that form).
  * Errors: DC_EINVAL (NULL pointers, k outside [1, 64]), DC_ENOMEM, DC_ECUDA.
  */
 dc_status dc_fspb_dose_batch(dc_plan* plan, const float* fluence, int32_t k, float* dose,

@@ -8,8 +8,8 @@
 // its voxels into the isocentre plane and walks, row by row, the union of the
 // lanes' ROI discs over the beamlet grid; each lane applies the exact ROI and
 // depth-range test of its own pair.  Per-beam partial doses are summed in
-// beam order afterwards.  The same traversal, with the evaluation replaced by
-// a counter or by a CSR store, gives the dose-deposition matrix.
+// beam order afterwards.  The same traversal, with the evaluation followed by a
+// CSR store, gives the dose-deposition matrix.
 //
 // Hot-loop choices: table indices come from a magic-constant rounding (no
 // float->int conversion, which would share the quarter-rate pipe with the
