@@ -24,6 +24,7 @@ void set_error(const std::string& msg) { g_last_error = msg; }
 
 dc_status cuda_fail(cudaError_t e, const char* what)
 {
+    cudaGetLastError();   // reported here: not again by a later call's launch check
     set_error(std::string(what) + ": " + cudaGetErrorName(e) + " (" + cudaGetErrorString(e) + ")");
     return e == cudaErrorMemoryAllocation ? DC_ENOMEM : DC_ECUDA;
 }
@@ -55,7 +56,9 @@ cudaError_t dev_malloc_bytes(void** p, size_t bytes)
             }
         }
     }
-    return cudaMalloc(p, bytes);
+    const cudaError_t e = cudaMalloc(p, bytes);
+    if (e != cudaSuccess) cudaGetLastError();   // the caller has it: not for a later call's launch check
+    return e;
 }
 
 template <typename T>
@@ -607,6 +610,7 @@ dc_status dc_fspb_destroy(dc_plan* plan)
     if (plan) {
         cudaStreamSynchronize(plan->stream);
         free_plan(plan);
+        cudaGetLastError();   // not reported here, nor by a later call's launch check
     }
     return DC_OK;
 }

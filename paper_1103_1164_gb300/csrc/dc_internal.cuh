@@ -193,6 +193,22 @@ dc_status cuda_fail(cudaError_t e, const char* what);
         if (e_ != cudaSuccess) return dc::cuda_fail(e_, #call);             \
     } while (0)
 
+// Launches a kernel and returns the status of this launch alone: cudaGetLastError
+// after <<<>>> would also give an error that another call has left on the thread.
+template <typename... Params, typename... Args>
+inline cudaError_t launch_kernel(void (*kern)(Params...), int grid, int block, size_t smem, cudaStream_t stream,
+                                 const Args&... args)
+{
+    cudaLaunchConfig_t c{};
+    c.gridDim = dim3(grid);
+    c.blockDim = dim3(block);
+    c.dynamicSmemBytes = smem;
+    c.stream = stream;
+    const cudaError_t e = cudaLaunchKernelEx(&c, kern, Params(args)...);
+    if (e == cudaSuccess) count_launches(1);
+    return e;
+}
+
 // kernel launchers (defined in the kernel translation units) ------------------
 cudaError_t launch_geometry(const dc_plan* p);         // once per plan: beamlet geometry, theta-blended A rows
 cudaError_t launch_smooth_factors(const dc_plan* p);   // smoothed density and the voxels' factors

@@ -2039,9 +2039,7 @@ cudaError_t launch_zeroed(const dc_plan* p, K kern, size_t sm, const Args&... ar
     if (e != cudaSuccess) return e;
     e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, p->device);
     if (e != cudaSuccess) return e;
-    kern<<<sms * (per_sm > 0 ? per_sm : 1), kThreads, sm, p->stream>>>(args...);
-    count_launches(1);
-    return cudaGetLastError();
+    return launch_kernel(kern, sms * (per_sm > 0 ? per_sm : 1), kThreads, sm, p->stream, args...);
 }
 
 // The same with the counter of d_work[1], which is cleared here.
@@ -2242,14 +2240,16 @@ cudaError_t launch_dose(const dc_plan* p, const float* fluence, int nf, int ldf,
     }
     if (p->part_cap < (size_t)p->n_beams * p->V) return cudaErrorInvalidValue;
     // the dose has a counter of its own, zeroed by the binning and by k_sum_beams
-    // after each pass: no clearing of 2 us before the smallest plans' 32
+    // after each pass: no clearing of 2 us before the smallest plans' 16.  A pass
+    // that does not get as far as its sum has it cleared here, or the next dose
+    // would find no work left and sum this one's partials.
     a.work = p->d_work + 2;
-    const cudaError_t e = run<kDose, 1>(p, a);
-    if (e != cudaSuccess) return e;
-    k_sum_beams<<<grid_for(p->V), 256, 0, p->stream>>>(p->d_part, p->d_cellof, p->n_beams, p->V, dose,
-                                                        p->d_work + 3);
-    count_launches(1);
-    return cudaGetLastError();
+    cudaError_t e = run<kDose, 1>(p, a);
+    if (e == cudaSuccess)
+        e = launch_kernel(k_sum_beams, grid_for(p->V), 256, 0, p->stream, p->d_part, p->d_cellof, p->n_beams, p->V, dose,
+                          p->d_work + 3);
+    if (e != cudaSuccess) cudaMemsetAsync(p->d_work + 3, 0, sizeof(int32_t), p->stream);
+    return e;
 }
 
 cudaError_t launch_count(const dc_plan* p, int32_t* counts)
@@ -2297,12 +2297,10 @@ cudaError_t launch_fill(const dc_plan* p, const int64_t* rowptr, int32_t* cols, 
     a.nf = 1;
     a.ldf = p->B;
     a.part = p->d_part;
-    cudaError_t e = run<kFill, 1>(p, a);
+    const cudaError_t e = run<kFill, 1>(p, a);
     if (e != cudaSuccess) return e;
-    k_sum_beams<<<grid_for(p->V), 256, 0, p->stream>>>(p->d_part, p->d_cellof, p->n_beams, p->V, dose,
-                                                        p->d_work + 3);
-    count_launches(1);
-    return cudaGetLastError();
+    return launch_kernel(k_sum_beams, grid_for(p->V), 256, 0, p->stream, p->d_part, p->d_cellof, p->n_beams, p->V, dose,
+                         p->d_work + 3);
 }
 
 cudaError_t launch_mark_patches(const dc_plan* p, const PatchTiles& t)

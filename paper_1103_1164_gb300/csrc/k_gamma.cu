@@ -234,6 +234,7 @@ struct GammaBuffers {
             g_busy.fetch_and(~(1u << slot));
         }
         for (void* p : ptrs) cudaFree(p);
+        cudaGetLastError();   // what failed has been reported: not for a later call's launch check
     }
     template <typename T>
     cudaError_t get(T** p, size_t n)
