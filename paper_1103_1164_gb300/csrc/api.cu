@@ -642,19 +642,22 @@ dc_status dc_fspb_list_entries(dc_plan* plan, int64_t* n)
     return DC_OK;
 }
 
-// Per-beam partial dose buffer of at least `need` floats.
-static dc_status ensure_part(dc_plan* p, size_t need)
+}  // extern "C"
+
+dc_status dc::ensure_part(dc_plan* p, size_t need)
 {
     if (need <= p->part_cap) return DC_OK;
     DC_CUDA(cudaStreamSynchronize(p->stream));
+    ++p->layout_gen;   // also if the allocation fails: no captured graph may use the freed buffer
     cudaFree(p->d_part);
     p->d_part = nullptr;
     p->part_cap = 0;
     DC_CUDA(dalloc(&p->d_part, need));
     p->part_cap = need;
-    ++p->layout_gen;
     return DC_OK;
 }
+
+extern "C" {
 
 static dc_status ensure_staging(dc_plan* p, size_t nflu, size_t ndose)
 {

@@ -94,6 +94,11 @@ dc_status refresh_args(dc_batch* bt)
     for (int i = 0; i < bt->n && !stale; ++i) stale = bt->gen[i] != bt->plans[i]->layout_gen;
     if (!stale) return DC_OK;
     bt->drop_graphs();
+    // a plan is without its partial doses after a call that found no memory for larger ones
+    for (dc_plan* p : bt->plans) {
+        const dc_status s = ensure_part(p, (size_t)p->n_beams * p->V);
+        if (s != DC_OK) return s;
+    }
     std::vector<DoseArgs>& args = bt->h_args;
     args.resize(bt->n);
     for (int j = 0; j < bt->n; ++j) {

@@ -193,6 +193,10 @@ dc_status cuda_fail(cudaError_t e, const char* what);
         if (e_ != cudaSuccess) return dc::cuda_fail(e_, #call);             \
     } while (0)
 
+// Per-beam partial dose buffer of at least `need` floats (freed, and the plan left
+// without one, if there is no memory for a larger one).
+dc_status ensure_part(dc_plan* p, size_t need);
+
 // Launches a kernel and returns the status of this launch alone: cudaGetLastError
 // after <<<>>> would also give an error that another call has left on the thread.
 template <typename... Params, typename... Args>

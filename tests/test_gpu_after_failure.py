@@ -73,3 +73,31 @@ def test_calls_after_a_failed_allocation(dc, many_units, fail):
         if w is not None and not np.array_equal(got, w):
             wrong.append(name)
     assert not wrong and not reported
+
+
+def test_batch_after_a_plan_lost_its_partial_doses(dc, monkeypatch):
+    # 64 vectors want a larger buffer of partial doses, whose allocation fails: the
+    # batch's captured graphs must not use the one that was freed for it
+    plans = [synth.small_plan(520 + j, n=(15, 16, 11), vox=0.25, n_beams=3, roi=2.0) for j in range(2)]
+    live = [dc.dc_fspb_create_from(p) for p in plans]
+    fluences = [p.fluence for p in plans]
+    want = [dc.dc_fspb_dose(dc.dc_fspb_create_from(p), p.fluence).reshape(-1) for p in plans]
+    for variant in range(3):
+        batch = dc.dc_fspb_batch_create(live)
+        dc.dc_fspb_batch_set_variant(batch, variant)
+        for fail_again in (False, True):
+            for density in (False, True):
+                for got, w in zip(dc.dc_fspb_batch_dose(batch, fluences, density=density), want):
+                    assert np.array_equal(got.reshape(-1), w)
+            # plan creation leaves room for one vector, the batch for no more
+            F = np.ones((64, live[0].n_beamlets), np.float32)
+            monkeypatch.setenv("DC_FSPB_FAIL_ALLOC_AT", "1")
+            with pytest.raises(dc.DcError) as ei:
+                dc.dc_fspb_dose_batch(live[0], F)
+            assert ei.value.status == dc.DC_ENOMEM
+            if fail_again:   # no memory for the batch either: an error, no launch
+                monkeypatch.setenv("DC_FSPB_FAIL_ALLOC_AT", "01")
+                with pytest.raises(dc.DcError) as ei:
+                    dc.dc_fspb_batch_dose(batch, fluences)
+                assert ei.value.status == dc.DC_ENOMEM
+            monkeypatch.delenv("DC_FSPB_FAIL_ALLOC_AT")
