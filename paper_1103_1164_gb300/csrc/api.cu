@@ -133,6 +133,29 @@ static void free_plan(dc_plan* p)
     delete p;
 }
 
+dc_status dc::ensure_part(dc_plan* p, size_t need)
+{
+    if (need <= p->part_cap) return DC_OK;
+    DC_CUDA(cudaStreamSynchronize(p->stream));
+    ++p->layout_gen;   // also if the allocation fails: no captured graph may use the freed buffer
+    cudaFree(p->d_part);
+    p->d_part = nullptr;
+    p->part_cap = 0;
+    DC_CUDA(dalloc(&p->d_part, need));
+    p->part_cap = need;
+    return DC_OK;
+}
+
+void dc::ensure_quads(dc_plan* p)
+{
+    if (p->d_quad || !p->coeffs.density_correction) return;
+    // (relaxed: the call may be part of a stream capture, which an allocation would end)
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    cudaThreadExchangeStreamCaptureMode(&mode);
+    if (dalloc(&p->d_quad, p->V) != cudaSuccess) p->d_quad = nullptr;
+    cudaThreadExchangeStreamCaptureMode(&mode);
+}
+
 extern "C" {
 
 const char* dc_last_error(void) { return g_last_error.c_str(); }
@@ -432,7 +455,7 @@ static dc_status create_impl(dc_plan* p, const float* ct, uint32_t flags)
     p->part_cap = nb * V;
     DC_CUDA(dalloc(&p->d_bcount, nb * V));
     DC_CUDA(dalloc(&p->d_lfac, nb * (V + 32)));
-    DC_CUDA(dalloc(&p->d_quad, V));
+    if (p->lateral_mode == DC_LATERAL_AXIS) ensure_quads(p);
     DC_CUDA(dalloc(&p->d_nfall, 1));
     DC_CUDA(dalloc(&p->d_chk, 1));
     DC_CUDA(cudaMemsetAsync(p->d_chk, 0, sizeof(int32_t), p->stream));
@@ -641,23 +664,6 @@ dc_status dc_fspb_list_entries(dc_plan* plan, int64_t* n)
     *n = s;
     return DC_OK;
 }
-
-}  // extern "C"
-
-dc_status dc::ensure_part(dc_plan* p, size_t need)
-{
-    if (need <= p->part_cap) return DC_OK;
-    DC_CUDA(cudaStreamSynchronize(p->stream));
-    ++p->layout_gen;   // also if the allocation fails: no captured graph may use the freed buffer
-    cudaFree(p->d_part);
-    p->d_part = nullptr;
-    p->part_cap = 0;
-    DC_CUDA(dalloc(&p->d_part, need));
-    p->part_cap = need;
-    return DC_OK;
-}
-
-extern "C" {
 
 static dc_status ensure_staging(dc_plan* p, size_t nflu, size_t ndose)
 {

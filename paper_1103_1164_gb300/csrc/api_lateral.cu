@@ -118,6 +118,7 @@ dc_status dc_fspb_set_lateral_mode(dc_plan* plan, int32_t mode)
         return bad("dc_fspb_set_lateral_mode: unknown mode");
     if (mode == DC_LATERAL_MLP && !plan->mlp_ready)
         return bad("dc_fspb_set_lateral_mode: the network form needs dc_fspb_set_surrogate first");
+    if (mode == DC_LATERAL_AXIS) ensure_quads(plan);
     plan->lateral_mode = mode;
     ++plan->layout_gen;
     if (plan->coeffs.density_correction && mode != DC_LATERAL_ISO) DC_CUDA(launch_lateral(plan));

@@ -43,7 +43,7 @@ struct dc_plan {
     int lateral_mode = 0;
     int precision = DC_PRECISION_FP32;   // arithmetic of the direct dose (dc_fspb_set_precision)
     float4* d_lfac = nullptr;        // [n_beams][V + 32]
-    float4* d_quad = nullptr;        // [V] density at a voxel and its +x, +y neighbours (axis stencil)
+    float4* d_quad = nullptr;        // [V] density at a voxel and its +x, +y neighbours (axis stencil; or null)
     float* d_leaf = nullptr;         // leaf sequences of dc_fluence_from_leaves (packed)
     size_t leaf_cap = 0;             // floats allocated at d_leaf
     uint2* d_mlp_frag = nullptr;     // BF16 B fragments of the surrogate network
@@ -196,6 +196,10 @@ dc_status cuda_fail(cudaError_t e, const char* what);
 // Per-beam partial dose buffer of at least `need` floats (freed, and the plan left
 // without one, if there is no memory for a larger one).
 dc_status ensure_part(dc_plan* p, size_t need);
+
+// The axis form's density quads (16 bytes per voxel), allocated when a plan first
+// takes that form; without memory for them its factors come from the volume.
+void ensure_quads(dc_plan* p);
 
 // Launches a kernel and returns the status of this launch alone: cudaGetLastError
 // after <<<>>> would also give an error that another call has left on the thread.

@@ -211,11 +211,13 @@ __global__ void __launch_bounds__(256) k_quads(const float* __restrict__ rho, in
     }
 }
 
-// Plain axis-stencil factors for every list entry: 48 taps of 8 densities each.
+// Plain axis-stencil factors for every list entry: 48 taps of 8 densities each,
+// from the quads or, for plans without them, from the volume (the same values).
 // Bound by the L1 data pipe (the lanes of a warp lie in several rows, so a load
 // touches several lines), hence few and wide loads: 205 us and 7.5 us for the quads
 // (97 x 91 x 71 voxels, 5 beams) against 378 us with eight loads of 4 bytes per tap and clamps.
-__global__ void __launch_bounds__(128) k_axis_factors(const PlanView P, const float4* __restrict__ quad,
+template <typename Density>
+__global__ void __launch_bounds__(128) k_axis_factors(const PlanView P, const Density D,
                                                       const int32_t* __restrict__ items,
                                                       const int64_t* __restrict__ base, float4* __restrict__ lfac)
 {
@@ -226,7 +228,7 @@ __global__ void __launch_bounds__(128) k_axis_factors(const PlanView P, const fl
         const BeamDev& bm = P.beams[beam_of(base, P.n_beams, e)];
         float rx, ry, rz;
         voxel_centre(P, v, rx, ry, rz);
-        lfac[e] = lateral_factors(P, axis_densities(P, RhoQuads{quad}, bm, rx, ry, rz));
+        lfac[e] = lateral_factors(P, axis_densities(P, D, bm, rx, ry, rz));
     }
 }
 
@@ -620,11 +622,14 @@ cudaError_t launch_lateral(const dc_plan* p)
     const PlanView P = p->view();
     int64_t total = (int64_t)p->n_beams * (p->V + 32);
     int g = (int)std::min<int64_t>((total + 127) / 128, 152 * 16);
-    if (p->lateral_mode == DC_LATERAL_AXIS) {
+    if (p->lateral_mode == DC_LATERAL_AXIS && !p->d_quad) {
+        k_axis_factors<<<g, 128, 0, p->stream>>>(P, RhoVolume{p->d_rho}, p->d_items, p->d_base, p->d_lfac);
+        count_launches(1);
+    } else if (p->lateral_mode == DC_LATERAL_AXIS) {
         const dc_grid& n = p->grid;
         const int gq = (int)std::min<int64_t>((p->V + 255) / 256, 152 * 64);
         k_quads<<<gq, 256, 0, p->stream>>>(p->d_rho, n.nx, n.ny, n.nz, p->d_quad);
-        k_axis_factors<<<g, 128, 0, p->stream>>>(P, p->d_quad, p->d_items, p->d_base, p->d_lfac);
+        k_axis_factors<<<g, 128, 0, p->stream>>>(P, RhoQuads{p->d_quad}, p->d_items, p->d_base, p->d_lfac);
         count_launches(2);
     } else if (p->lateral_mode == DC_LATERAL_MLP) {
         cudaError_t e = cudaMemsetAsync(p->d_nfall, 0, sizeof(int32_t), p->stream);
