@@ -702,7 +702,9 @@ dc_status dc_fspb_dose_batch(dc_plan* plan, const float* fluence, int32_t k, flo
         DC_CUDA(dc::dev_malloc(&plan->d_sp_fp, (size_t)plan->B * 64 * sizeof(uint16_t)));
         plan->sp_fp_cap = (size_t)plan->B * 64;
     }
-    const size_t need_pack = k > 1 && !tc ? (size_t)plan->B * dose_pass_width(k) : 0;
+    // (in the tensor-core form too: a later call in FP32 then allocates nothing, as
+    // inside a stream capture)
+    const size_t need_pack = k > 1 ? (size_t)plan->B * (tc ? 64 : dose_pass_width(k)) : 0;
     if (plan->flupack_cap < need_pack) {
         if (plan->d_flupack) cudaFree(plan->d_flupack);
         plan->d_flupack = nullptr;
