@@ -115,7 +115,7 @@ struct DoseArgs {
     float* part;            // dose: per-beam partial dose [n_beams][V][NF], written where the beam lists the voxel
     const int32_t* cell;    // [n_beams][V]: the voxel's cell in the beam's list (k_bin.cu), -1 if it is not listed
     const uint4* fpack;     // dose, tensor-core form: the fluences as BF16 [B][64] (zero past nf)
-    const float4* fpack32;  // dose, several vectors: the fluences [B][NF] (zero past nf)
+    const float4* fpack32;  // dose, several vectors, many units: the fluences [B][NF] (zero past nf)
     int32_t* bcount;        // count: per-beam pair counts [n_beams][V]; fill reads them
     int32_t* count_out;     // dose with one fluence vector: where to record the same counts (or null)
     const int64_t* rowptr;  // fill

@@ -1077,26 +1077,25 @@ __global__ void __launch_bounds__(kThreads, NV <= 2 ? 4 : (NV == 3 ? 3 : 2)) k_c
 }
 
 // ---------------------------------------------------------------------------
-// Several fluence vectors in one FP32 pass.  Per unit of 32 voxels and 16
+// Several fluence vectors in one FP32 pass.  Per unit of 32 voxels and 16 or 32
 // beamlets, the pair values D[16][32] are evaluated a voxel per lane into shared
 // memory (zero outside the pairs), and Y[32][NF] += D F is a register-tiled
 // product, 8 voxels x 2 or 4 vectors per lane, so a beamlet costs a lane 3
-// shared-memory vector loads for its 16 or 32 multiply-adds.  64 vectors take
-// two warps per unit, each evaluating every other beamlet and holding half of
-// the vectors.  Each sum runs over the beamlets in order, as the single-vector
-// pass's.  The fluences come packed as [B][NF] (zero past nf), the partial doses
-// go out as [n_beams][V][NF], whole lines per voxel.  Bound by issue slots and,
+// shared-memory vector loads for its 16 or 32 multiply-adds.  64 vectors, and
+// fewer on plans of few units, take two warps per unit, each evaluating every
+// other beamlet and holding half of the vectors (or, of 16, half of the voxels).
+// Each sum runs over the beamlets in order, as the single-vector
+// pass's.  The fluences come packed as [B][NF] (zero past nf), or as they are given
+// on plans of few units (no packing launch of 3 us), the partial doses go out as [n_beams][V][NF], whole lines per voxel.  Bound by issue slots and,
 // with the 24 or 32 warps per SM that the accumulators leave, by the latency of
 // the table loads: a call of 64 vectors on the thorax plan (516 M pairs) takes
 // 6.7 ms with one warp per unit, which leaves 16 warps, 6.3 ms with two, and took
 // 9.45 ms with a vector load per four multiply-adds.  32 vectors: 6.4 -> 4.4 ms,
-// 11 vectors: 4.0 -> 3.5 ms.
-constexpr int kMultiRows = 16;
-
-template <int NF>
+// 11 vectors: 4.0 -> 3.5 ms.  Few units: see run_multi.
+template <int NF, bool FEW>
 constexpr int multi_ctas()
 {
-    return NF == 16 ? 4 : 3;
+    return NF == 16 || FEW ? 4 : 3;
 }
 
 // All threads of a unit's warps (pair `unit` of the CTA's warps, or one warp).
@@ -1104,29 +1103,36 @@ template <int WPU>
 __device__ __forceinline__ void unit_sync(int unit)
 {
     if (WPU == 1) __syncwarp();
-    else asm volatile("bar.sync %0, 64;" ::"r"(unit + 1) : "memory");
+    else asm volatile("bar.sync %0, %1;" ::"r"(unit + 1), "n"(32 * WPU) : "memory");
 }
 
-template <int NF, bool MERGED, int LAT>
-__global__ void __launch_bounds__(kThreads, multi_ctas<NF>()) k_dose_multi(const DoseArgs a)
+// FEW: the form of plans with few units (run_multi)
+template <int NF, bool FEW, bool MERGED, int LAT>
+__global__ void __launch_bounds__(kThreads, multi_ctas<NF, FEW>()) k_dose_multi(const DoseArgs a)
 {
-    constexpr int WPU = NF == 64 ? 2 : 1;    // warps per unit
-    constexpr int NW = NF / WPU;             // vectors per warp
+    constexpr int WPU = NF == 64 || FEW ? 2 : 1;        // warps per unit
+    constexpr int SV = NF / 16 < WPU ? NF / 16 : WPU;   // a unit's warps share the vectors SV ways ...
+    constexpr int SX = WPU / SV;                        // ... and the voxels SX ways
+    constexpr int NW = NF / SV;              // vectors per warp
     constexpr int VP = NW / 8;               // vectors per lane: 2 or 4
+    constexpr int VX = 8 / SX;               // voxels per lane
     constexpr int kUnits = kWarps / WPU;     // units per CTA
+    constexpr int kRows = FEW ? 32 : 16;     // beamlets per chunk
     extern __shared__ float4 smem[];
     __shared__ int64_t s_base[kMaxBeams + 1];
-    __shared__ float4 s_row[kUnits][3 * kMultiRows];
-    __shared__ float4 s_d[kUnits][kMultiRows * 8];
-    __shared__ float4 s_f[kUnits][kMultiRows * NF / 4];
-    __shared__ uint32_t s_in[kUnits][kMultiRows];   // which of the 32 voxels are pairs (non-finite fluences only)
+    __shared__ float4 s_row[kUnits][3 * kRows];
+    __shared__ float4 s_d[kUnits][kRows * 8];
+    __shared__ float4 s_f[kUnits][kRows * NF / 4];
+    __shared__ uint32_t s_in[kUnits][kRows];   // which of the 32 voxels are pairs (non-finite fluences only)
     __shared__ RowWindows s_win[kWarps];
     __shared__ int s_w[kUnits], s_bad[kUnits];
     const PlanView& P = a.P;
     const int64_t V = (int64_t)P.nx * P.ny * P.nz;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int unit = warp / WPU, half = warp % WPU, ut = threadIdx.x % (32 * WPU);
-    const int vg = lane >> 3, fg = lane & 7;   // the lane's voxels 8 vg .. 8 vg + 7, vectors VP fg .. of the warp's
+    const int unit = warp / WPU, part = warp % WPU, ut = threadIdx.x % (32 * WPU);
+    const int nw0 = NW * (part % SV);          // the warp's first vector
+    const int fg = lane & 7;                   // the lane's vectors VP fg .. of the warp's
+    const int vx0 = (32 / SX) * (part / SV) + VX * (lane >> 3);   // the lane's first voxel
     if (!MERGED)
         for (int q = threadIdx.x; q < 2 * P.w_n; q += blockDim.x) smem[q] = __ldg(P.water + q);
     for (int q = threadIdx.x; q <= P.n_beams; q += blockDim.x) s_base[q] = a.base[q];
@@ -1174,20 +1180,20 @@ __global__ void __launch_bounds__(kThreads, multi_ctas<NF>()) k_dose_multi(const
             ln.cw1 = lf.z;
             ln.cw2 = lf.w;
         }
-        float acc[8][VP];
+        float acc[VX][VP];
 #pragma unroll
-        for (int j = 0; j < 8; ++j)
+        for (int j = 0; j < VX; ++j)
 #pragma unroll
             for (int q = 0; q < VP; ++q) acc[j][q] = 0.f;
         for (int nb = n0; nb <= n1; nb += 32) {
             const int places = row_windows(P, box, win, nb, n1, __ldg(&bm.M), __ldg(&bm.first), __ldg(&bm.half_fx),
                                            __ldg(&bm.half_fy), lane);
-            for (int q0 = 0; q0 < places; q0 += kMultiRows) {
-                const int nq = min(kMultiRows, places - q0);
+            for (int q0 = 0; q0 < places; q0 += kRows) {
+                const int nq = min(kRows, places - q0);
                 int ib = 0;
                 if (lane < nq) ib = (int)DC_GUARD(P, win.base[window_row(win, q0 + lane)] + q0 + lane, P.B, 5);
                 unit_sync<WPU>(unit);   // the last chunk's product has read its operands
-                if (half == 0 && lane < nq) {
+                if (part == 0 && lane < nq) {
                     const float4* src = reinterpret_cast<const float4*>(P.bl) + 4u * (uint32_t)ib;
                     srow[3 * lane] = __ldg(src);
                     srow[3 * lane + 1] = __ldg(src + 1);
@@ -1195,11 +1201,17 @@ __global__ void __launch_bounds__(kThreads, multi_ctas<NF>()) k_dose_multi(const
                 }
                 bool finite = true;
 #pragma unroll
-                for (int t = 0; t < kMultiRows * NF / 4; t += 32 * WPU) {
-                    const int j = (t + ut) / (NF / 4);
+                for (int t = 0; t < kRows * NF / 4; t += 32 * WPU) {
+                    const int j = (t + ut) / (NF / 4), n4 = (t + ut) % (NF / 4);
                     const int i = __shfl_sync(0xffffffffu, ib, j);
                     if (j < nq) {
-                        const float4 f = __ldg(a.fpack32 + (size_t)i * (NF / 4) + (t + ut) % (NF / 4));
+                        float4 f;
+                        if constexpr (FEW) {
+                            const auto at = [&](int n) { return n < a.nf ? __ldg(a.fluence + (size_t)n * a.ldf + i) : 0.f; };
+                            f = make_float4(at(4 * n4), at(4 * n4 + 1), at(4 * n4 + 2), at(4 * n4 + 3));
+                        } else {
+                            f = __ldg(a.fpack32 + (size_t)i * (NF / 4) + n4);
+                        }
                         sf[t + ut] = f;
                         finite = finite && fabsf(f.x) <= 3.402823466e38f && fabsf(f.y) <= 3.402823466e38f &&
                                  fabsf(f.z) <= 3.402823466e38f && fabsf(f.w) <= 3.402823466e38f;
@@ -1209,8 +1221,8 @@ __global__ void __launch_bounds__(kThreads, multi_ctas<NF>()) k_dose_multi(const
                 if (WPU > 1 && !finite && lane == 0) s_bad[unit] = 1;
                 unit_sync<WPU>(unit);
                 const bool bad = WPU > 1 ? s_bad[unit] != 0 : !finite;
-#pragma unroll 2
-                for (int m = half; m < nq; m += WPU) {
+#pragma unroll (FEW && NF == 16 ? 4 : 2)
+                for (int m = part; m < nq; m += WPU) {
                     const uint32_t i = (uint32_t)__shfl_sync(0xffffffffu, ib, m);
                     const float4* rq = srow + 3 * m;
                     const PairTest pt = pair_test(P, ln, rq[0], rq[1], rq[2]);
@@ -1225,15 +1237,22 @@ __global__ void __launch_bounds__(kThreads, multi_ctas<NF>()) k_dose_multi(const
                 unit_sync<WPU>(unit);
 #pragma unroll 4
                 for (int m = 0; m < nq; ++m) {
-                    const float4 d0 = s_d[unit][m * 8 + 2 * vg], d1 = s_d[unit][m * 8 + 2 * vg + 1];
-                    const float d[8] = {d0.x, d0.y, d0.z, d0.w, d1.x, d1.y, d1.z, d1.w};
-                    float f[VP];
+                    float d[VX], f[VP];
+#pragma unroll
+                    for (int j = 0; j < VX; j += 4) {
+                        const float4 g = *reinterpret_cast<const float4*>(sd + m * 32 + vx0 + j);
+                        d[j] = g.x;
+                        d[j + 1] = g.y;
+                        d[j + 2] = g.z;
+                        d[j + 3] = g.w;
+                    }
+                    const float* fm = reinterpret_cast<const float*>(sf) + m * NF + nw0 + VP * fg;
                     if (VP == 2) {
-                        const float2 g = reinterpret_cast<const float2*>(sf + m * (NF / 4))[fg];
+                        const float2 g = *reinterpret_cast<const float2*>(fm);
                         f[0] = g.x;
                         f[1] = g.y;
                     } else {
-                        const float4 g = sf[m * (NF / 4) + 8 * half + fg];
+                        const float4 g = *reinterpret_cast<const float4*>(fm);
                         f[0] = g.x;
                         f[1] = g.y;
                         f[VP - 2] = g.z;
@@ -1241,14 +1260,14 @@ __global__ void __launch_bounds__(kThreads, multi_ctas<NF>()) k_dose_multi(const
                     }
                     if (!bad) {
 #pragma unroll
-                        for (int j = 0; j < 8; ++j)
+                        for (int j = 0; j < VX; ++j)
 #pragma unroll
                             for (int q = 0; q < VP; ++q) acc[j][q] = fmaf(f[q], d[j], acc[j][q]);
                     } else {
                         // an infinite or NaN fluence reaches the beamlet's own pairs only
-                        const uint32_t in = s_in[unit][m] >> (8 * vg);
+                        const uint32_t in = s_in[unit][m] >> vx0;
 #pragma unroll
-                        for (int j = 0; j < 8; ++j)
+                        for (int j = 0; j < VX; ++j)
 #pragma unroll
                             for (int q = 0; q < VP; ++q)
                                 if ((in >> j) & 1u) acc[j][q] = fmaf(f[q], d[j], acc[j][q]);
@@ -1257,14 +1276,14 @@ __global__ void __launch_bounds__(kThreads, multi_ctas<NF>()) k_dose_multi(const
             }
         }
 #pragma unroll
-        for (int j = 0; j < 8; ++j) {
-            const int v = __shfl_sync(0xffffffffu, vi, 8 * vg + j);
-            if (v < 0 || NW * half + VP * fg >= a.nf) continue;
-            float* out = a.part + ((size_t)b * V + v) * NF + NW * half;
+        for (int j = 0; j < VX; ++j) {
+            const int v = __shfl_sync(0xffffffffu, vi, vx0 + j);
+            if (v < 0 || nw0 + VP * fg >= a.nf) continue;
+            float* out = a.part + ((size_t)b * V + v) * NF + nw0 + VP * fg;
             if (VP == 2)
-                reinterpret_cast<float2*>(out)[fg] = make_float2(acc[j][0], acc[j][1]);
+                *reinterpret_cast<float2*>(out) = make_float2(acc[j][0], acc[j][1]);
             else
-                reinterpret_cast<float4*>(out)[fg] = make_float4(acc[j][0], acc[j][1], acc[j][VP - 2], acc[j][VP - 1]);
+                *reinterpret_cast<float4*>(out) = make_float4(acc[j][0], acc[j][1], acc[j][VP - 2], acc[j][VP - 1]);
         }
     }
 }
@@ -2098,18 +2117,38 @@ __global__ void __launch_bounds__(256) k_pack_fluence_bf16(const float* __restri
     }
 }
 
-// One FP32 pass of NF fluence vectors (fluence packed as [B][NF]).
+template <int NF, bool FEW>
+cudaError_t launch_multi(const dc_plan* p, const DoseArgs& a)
+{
+    const bool item = p->coeffs.density_correction && p->lateral_mode != DC_LATERAL_ISO;
+    auto kern = p->merged ? (item ? k_dose_multi<NF, FEW, true, kItem> : k_dose_multi<NF, FEW, true, kIso>)
+                          : (item ? k_dose_multi<NF, FEW, false, kItem> : k_dose_multi<NF, FEW, false, kIso>);
+    return launch_units(p, kern, p->merged ? 0 : 2 * sizeof(float4) * p->coeffs.w_n, a);
+}
+
+// One FP32 pass of NF fluence vectors.  Up to 128 units per SM take the form of few
+// units: there a call is bound by one unit's chain of loads and barriers, so two
+// warps share a unit, in chunks of 32 beamlets instead of 16.  Calls of 2 vectors (a
+// load per four multiply-adds | packed fluences, a warp per unit | this form):
+// 252 units of 452 beamlets 170 | 197 | 128 us, 1,512 of 314 86 | 103 | 66, 3,420 of
+// 50 50 | 56 | 37, of 314 109 | 133 | 110, 9,828 of 50 60 | 59 | 47; 20 vectors: 252 of
+// 452 175 | 216 | 138, 3,420 of 314 165 | 125 | 132.  At 19,656 units a warp per unit
+// takes 336 us and two 351 (314 beamlets), 524 and 502 (452 beamlets).
 template <int NF>
 cudaError_t run_multi(const dc_plan* p, const DoseArgs& a, float* dose, int64_t ldd)
 {
-    const bool item = p->coeffs.density_correction && p->lateral_mode != DC_LATERAL_ISO;
-    auto kern = p->merged ? (item ? k_dose_multi<NF, true, kItem> : k_dose_multi<NF, true, kIso>)
-                          : (item ? k_dose_multi<NF, false, kItem> : k_dose_multi<NF, false, kIso>);
-    const size_t sm = p->merged ? 0 : 2 * sizeof(float4) * p->coeffs.w_n;
-    k_pack_fluence<<<dim3((p->B + 31) / 32, (NF + 31) / 32), 256, 0, p->stream>>>(
-        a.fluence, a.nf, a.ldf, p->B, NF, reinterpret_cast<float*>(p->d_flupack));
-    count_launches(1);
-    cudaError_t e = launch_units(p, kern, sm, a);
+    int sms = 0;
+    cudaError_t e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, p->device);
+    if (e != cudaSuccess) return e;
+    const int64_t units = (int64_t)p->n_beams * ((p->V + 31) / 32);   // at most
+    if (NF < 64 && units <= (int64_t)sms * 128) {
+        e = launch_multi<NF, NF < 64>(p, a);
+    } else {
+        k_pack_fluence<<<dim3((p->B + 31) / 32, (NF + 31) / 32), 256, 0, p->stream>>>(
+            a.fluence, a.nf, a.ldf, p->B, NF, reinterpret_cast<float*>(p->d_flupack));
+        count_launches(1);
+        e = launch_multi<NF, false>(p, a);
+    }
     if (e != cudaSuccess) return e;
     k_sum_vectors<NF><<<grid_for(p->V * 8), 256, 0, p->stream>>>(reinterpret_cast<const float4*>(p->d_part), p->d_cellof,
                                                                  p->n_beams, a.nf, p->V, dose, ldd);
