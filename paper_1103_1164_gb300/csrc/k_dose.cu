@@ -2082,10 +2082,12 @@ cudaError_t run_variant(const dc_plan* p, const DoseArgs& a)
         // 45-76 us -> 35-59, and with 452 beamlets per window 256 -> 137.  With so
         // many (ROI area / beamlet area) it pays up to 32: 3,600 units 250 -> 155,
         // 4,800 150 -> 130; with 113 to 314 it does not (4,200 units 68 -> 78, 4,800
-        // 101 -> 116).
+        // 101 -> 116).  With few a warp is soon done: windows of 3 to 7 beamlets take
+        // 18-21 us from 2,000 to 4,000 units with a warp per unit and 25-27 at 2,000
+        // with a CTA, which pays up to some 1,200 (15-19 us), hence 8 units per SM.
         const double window = 3.1416 * p->coeffs.roi_radius * p->coeffs.roi_radius / ((double)p->bx * p->by);
         // (three CTAs or more fit with water tables of up to 24 KB)
-        if (sm <= 24 * 1024 && units <= (int64_t)sms * (window >= 400. ? 32 : 16))
+        if (sm <= 24 * 1024 && units <= (int64_t)sms * (window >= 400. ? 32 : (window >= 10. ? 16 : 8)))
             return launch_zeroed(p, k_dose_small<MERGED, LAT, PREC>, sm, a);
         // no more units than warps with 4 CTAs per SM
         if (units <= (int64_t)sms * 4 * kWarps)
