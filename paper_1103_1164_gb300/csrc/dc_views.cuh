@@ -126,11 +126,12 @@ struct DoseArgs {
     const int64_t* base;    // [n_beams + 1]
     int32_t* work;          // [0] work units, [1] counter
     // backward pass with respect to the commissioning tables: voxel weights
-    // [V] and the gradients [4][w_n], [4][f_n], [2]
+    // [V], the gradients [4][w_n], [4][f_n], [2] and log2 of the work items per unit
     const float* wv;
     float* g_water;
     float* g_dens;
     float* g_corr;
+    int grad_shift;
 };
 
 }  // namespace dc

@@ -40,11 +40,6 @@ constexpr int kRingLd = kRing + 1;
 constexpr int row_max(int mode, int nf = 1) { return mode == 2 || nf > 32 ? 16 : 32; }
 
 enum Mode { kDose = 0, kFill = 2, kGrad = 3 };
-// work items per unit of the backward pass, whose phantoms have few units (a 60^3
-// grid: 6,750 for 4,864 warps, so whole units ran in two rounds).  A single call on
-// that grid: 385 us with 1 item, 254 with 2, 200 with 4, 220 with 8; 30^3: 225, 156,
-// 121, 106; 72^3, two beams: 390, 300, 267, 283.
-constexpr int kGradSplit = 4;
 
 // PREC 2, the tensor-core form of the multi-fluence dose (64 vectors): per
 // warp and chunk of 16 beamlets, Y[32 voxels][64] += D[32][16] F[16][64] as
@@ -283,7 +278,7 @@ __device__ __forceinline__ void penumbra_du(float ax, float u, float x0, float& 
 // segment in registers and adds them to the CTA's bins when the segment changes:
 // with eight shared-memory atomics per pair, contended by the lanes of a warp
 // (whose depths span a few samples), they were what bound the kernel: a call on a
-// 60^3 slab (7.5 M pairs) took 652 us, now 160, kGradSplit included.
+// 60^3 slab (7.5 M pairs) took 652 us, now 160, four work items per unit included.
 struct WaterSums {
     int j;
     float a0[4], a1[4];
@@ -500,7 +495,8 @@ __device__ __forceinline__ void flush_stage(const DoseArgs& a, const int2* st, i
 template <int MODE, int NF, bool MERGED, int LAT, int PREC = 0>
 __device__ __forceinline__ void process_unit(const DoseArgs& a, const int32_t vi, const int64_t e0, const int b,
                                              const float4* __restrict__ sW, int2* sst, float4* srow,
-                                             const int lane, uint32_t* stc = nullptr, const int split = 0)
+                                             const int lane, uint32_t* stc = nullptr, const int split = 0,
+                                             const int splits = 1)
 {
     // the tensor-core form of 64 fluence vectors; its pair values in FP32
     // exponentials like the plain form
@@ -570,8 +566,8 @@ __device__ __forceinline__ void process_unit(const DoseArgs& a, const int32_t vi
     }
     const int wnlo = __reduce_min_sync(0xffffffffu, nlo);
     const int wnhi = __reduce_max_sync(0xffffffffu, nhi);
-    // (the backward pass takes every kGradSplit-th row of a work item's window)
-    for (int n = wnlo + (MODE == kGrad ? split : 0); n <= wnhi; n += MODE == kGrad ? kGradSplit : 1) {
+    // (a work item of the backward pass takes every splits-th row of its unit's window)
+    for (int n = wnlo + (MODE == kGrad ? split : 0); n <= wnhi; n += MODE == kGrad ? splits : 1) {
         const float dc_ = cc - (-hfy + (n + 0.5f) * P.by);
         const float h2 = rw * rw - dc_ * dc_;
         int mlo = INT_MAX, mhi = INT_MIN;
@@ -790,19 +786,19 @@ __global__ void __launch_bounds__(kThreads, MINB) k_pairs(const DoseArgs a)
     for (int q = threadIdx.x; q <= P.n_beams; q += blockDim.x) s_base[q] = a.base[q];
     __syncthreads();
     const int total = a.work[0];
-    constexpr int kItems = MODE == kGrad ? kGradSplit : 1;   // work items per unit
+    const int shift = MODE == kGrad ? a.grad_shift : 0;   // 1 << shift work items per unit
 
     for (;;) {
         int w = 0;
         if (lane == 0) w = atomicAdd(a.work + 1, 1);
         w = __shfl_sync(0xffffffffu, w, 0);
-        if (w / kItems >= total) break;
-        const int64_t e0 = (int64_t)DC_GUARD(P, w / kItems, (s_base[P.n_beams] + 31) / 32, 4) * 32;
+        if (w >> shift >= total) break;
+        const int64_t e0 = (int64_t)DC_GUARD(P, w >> shift, (s_base[P.n_beams] + 31) / 32, 4) * 32;
         int b = 0;
         while (b + 1 < P.n_beams && s_base[b + 1] <= e0) ++b;
         const int32_t vi = __ldg(a.items + e0 + lane);
         process_unit<MODE, NF, MERGED, LAT, PREC>(a, vi, e0, b, sW, sst, s_row[warp], lane,
-                                                  TC ? s_tc[TC ? warp : 0] : nullptr, w % kItems);
+                                                  TC ? s_tc[TC ? warp : 0] : nullptr, w & ((1 << shift) - 1), 1 << shift);
     }
     if (MODE == kGrad) {
         __syncthreads();
@@ -2069,6 +2065,14 @@ cudaError_t launch_units(const dc_plan* p, K kern, size_t sm, const Args&... arg
     return e != cudaSuccess ? e : launch_zeroed(p, kern, sm, args...);
 }
 
+// The plan's work units at most (voxels outside a beam have none), and the beamlets
+// of a window (ROI area / beamlet area), by which launches choose their form.
+int64_t most_units(const dc_plan* p) { return (int64_t)p->n_beams * ((p->V + 31) / 32); }
+double window_beamlets(const dc_plan* p)
+{
+    return 3.1416 * p->coeffs.roi_radius * p->coeffs.roi_radius / ((double)p->bx * p->by);
+}
+
 template <int MODE, int NF, bool MERGED, int LAT, int PREC = 0>
 cudaError_t run_variant(const dc_plan* p, const DoseArgs& a)
 {
@@ -2077,15 +2081,15 @@ cudaError_t run_variant(const dc_plan* p, const DoseArgs& a)
         int sms = 0;
         const cudaError_t e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, p->device);
         if (e != cudaSuccess) return e;
-        const int64_t units = (int64_t)p->n_beams * ((p->V + 31) / 32);   // at most (voxels outside a beam have none)
+        const int64_t units = most_units(p);
         // A CTA per unit up to 16 units per SM: single calls with 405 to 2,400 units
         // 45-76 us -> 35-59, and with 452 beamlets per window 256 -> 137.  With so
-        // many (ROI area / beamlet area) it pays up to 32: 3,600 units 250 -> 155,
+        // many it pays up to 32: 3,600 units 250 -> 155,
         // 4,800 150 -> 130; with 113 to 314 it does not (4,200 units 68 -> 78, 4,800
         // 101 -> 116).  With few a warp is soon done: windows of 3 to 7 beamlets take
         // 18-21 us from 2,000 to 4,000 units with a warp per unit and 25-27 at 2,000
         // with a CTA, which pays up to some 1,200 (15-19 us), hence 8 units per SM.
-        const double window = 3.1416 * p->coeffs.roi_radius * p->coeffs.roi_radius / ((double)p->bx * p->by);
+        const double window = window_beamlets(p);
         // (three CTAs or more fit with water tables of up to 24 KB)
         if (sm <= 24 * 1024 && units <= (int64_t)sms * (window >= 400. ? 32 : (window >= 10. ? 16 : 8)))
             return launch_zeroed(p, k_dose_small<MERGED, LAT, PREC>, sm, a);
@@ -2142,7 +2146,7 @@ cudaError_t run_multi(const dc_plan* p, const DoseArgs& a, float* dose, int64_t 
     int sms = 0;
     cudaError_t e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, p->device);
     if (e != cudaSuccess) return e;
-    const int64_t units = (int64_t)p->n_beams * ((p->V + 31) / 32);   // at most
+    const int64_t units = most_units(p);
     if (NF < 64 && units <= (int64_t)sms * 128) {
         e = launch_multi<NF, NF < 64>(p, a);
     } else {
@@ -2377,6 +2381,20 @@ cudaError_t launch_dose_vjp(const dc_plan* p, const float* fluence, const float*
     if (e == cudaSuccess) e = cudaMemsetAsync(g_dens, 0, sizeof(float) * 4 * (size_t)p->coeffs.f_n, p->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(g_corr, 0, sizeof(float) * 2, p->stream);
     if (e != cudaSuccess) return e;
+    // Work items per unit: 4 or 2 where the units do not fill the GPU several times
+    // over (a 60^3 phantom has 6,750 for 4,864 warps), and for longer the more
+    // beamlets a window holds; each item repeats the unit's set-up and the sums at its
+    // end.  With 1 | 2 | 4: 844 units 201 | 132 | 98 us, 6,750 (314 beamlets) 575 | 348 |
+    // 254, 27,000 (28) 179 | 176 | 203, 62,500 (452) 1,560 | 1,183 | 1,108, 64,000 (78)
+    // 442 | 430 | 497, 113,910 (3) 120 | 160 | 236, 442,368 (314, thorax plan) 11.6 |
+    // 12.0 | 12.9 ms.
+    int sms = 0;
+    e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, p->device);
+    if (e != cudaSuccess) return e;
+    const int64_t units = most_units(p);
+    const double window = window_beamlets(p);
+    a.grad_shift = units <= (int64_t)sms * (window >= 400. ? 480 : (window >= 100. ? 160 : 100)) ? 2
+                   : (units <= (int64_t)sms * 480 ? 1 : 0);
     return run_variant<kGrad, 1, false, kIso>(p, a);
 }
 
