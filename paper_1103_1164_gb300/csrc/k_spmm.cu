@@ -485,14 +485,12 @@ __global__ void __launch_bounds__(kSpmmThreads) k_spmm(const SpmmArgs a)
 }
 
 // Y[v][q] = sum over beams of the partial rows, in beam order, with
-// Neumaier-compensated summation.  G lanes per voxel, as few as hold its k columns
-// two by two, so that row reads are whole lines and lanes do not idle: they look up
-// the voxel's list positions in G beams at once, one voxel ahead (that lookup's
-// latency overlaps the sums), then add the partial rows (lane l: columns 2l,
-// 2l + 1).  With a warp per voxel whatever the k: 196 us for k = 21 on 830 k voxels
-// and 5 beams, now 115; k = 8, 1.57 M voxels, 9 beams: 443 -> 161; k = 64 and 33
-// stay (357 -> 351, 508 -> 506).  Loading 3 to 8 beams' rows before adding any was
-// slower for k > 32 (373 to 500 us at k = 64).
+// Neumaier-compensated summation.  Up to 32 columns: G lanes per voxel, as few as
+// hold its k columns two by two, so that row reads are whole lines and lanes do not
+// idle: they look up the voxel's list positions in G beams at once, one voxel ahead
+// (that lookup's latency overlaps the sums), then add the partial rows (lane l:
+// columns 2l, 2l + 1).  With a warp per voxel whatever the k: 196 us for k = 21 on
+// 830 k voxels and 5 beams, now 115; k = 8, 1.57 M voxels, 9 beams: 443 -> 161.
 __device__ __forceinline__ void neumaier_add(float& s, float& c, float x)
 {
     const float t = s + x;
@@ -544,11 +542,49 @@ __global__ void __launch_bounds__(256) k_spmm_reduce(const float* __restrict__ P
     }
 }
 
+// The same for more than 32 columns: a warp per voxel, whose lanes look up two beams
+// each, so that there is no loop over groups of beams; with it (32 lanes of the kernel
+// above) the whole product took 75 us instead of 71 at k = 64 on 360 k voxels and 2
+// beams, most of them unlisted.  Loading 3 to 8 beams' rows before adding any was
+// slower (357 -> 373 to 500 us at k = 64, 9 beams), 9,728 blocks are better than 4,096
+// (1,368 -> 1,323 us for the product on the thorax plan).
+__global__ void __launch_bounds__(256) k_spmm_reduce_wide(const float* __restrict__ P, const int32_t* __restrict__ inv,
+                                                          int n_beams, int64_t V, int k, float* __restrict__ Y)
+{
+    const int lane = threadIdx.x & 31, q = 2 * lane;
+    const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    int64_t v = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
+    const auto lookup = [&](int64_t u, int32_t& a, int32_t& b) {   // at most 64 beams
+        a = u < V && lane < n_beams ? __ldg(inv + (size_t)lane * V + u) : -1;
+        b = u < V && lane + 32 < n_beams ? __ldg(inv + (size_t)(lane + 32) * V + u) : -1;
+    };
+    int32_t na, nb;
+    lookup(v, na, nb);
+    for (; v < V; v += nwarps) {
+        const int32_t pa = na, pb = nb;
+        lookup(v + nwarps, na, nb);
+        float s0 = 0.f, c0 = 0.f, s1 = 0.f, c1 = 0.f;
+#pragma unroll 4
+        for (int b = 0; b < n_beams; ++b) {
+            const int32_t pos = __shfl_sync(0xffffffffu, b < 32 ? pa : pb, b & 31);
+            if (pos < 0) continue;
+            const float* row = P + (size_t)pos * k;
+            if (q < k) neumaier_add(s0, c0, __ldg(row + q));
+            if (q + 1 < k) neumaier_add(s1, c1, __ldg(row + q + 1));
+        }
+        float* y = Y + (size_t)v * k;
+        if (q < k) y[q] = s0 + c0;
+        if (q + 1 < k) y[q + 1] = s1 + c1;
+    }
+}
+
+constexpr int kReduceBlocks = 152 * 64;
+
 template <int G>
 cudaError_t reduce_launch(cudaStream_t s, const float* P, const int32_t* inv, int n_beams, int64_t V, int k, float* Y)
 {
     const int64_t blocks = (V * G + 255) / 256;
-    const int grid = (int)std::min<int64_t>(blocks, 152 * 64);
+    const int grid = (int)std::min<int64_t>(blocks, kReduceBlocks);
     // pairs of columns as 8-byte words where every row starts on one
     if (k % 2 == 0 && ((reinterpret_cast<uintptr_t>(P) | reinterpret_cast<uintptr_t>(Y)) & 7) == 0)
         k_spmm_reduce<G, true><<<grid, 256, 0, s>>>(P, inv, n_beams, V, k, Y);
@@ -561,7 +597,9 @@ cudaError_t reduce_launch(cudaStream_t s, const float* P, const int32_t* inv, in
 cudaError_t spmm_reduce(cudaStream_t s, const float* P, const int32_t* inv, int n_beams, int64_t V, int k, float* Y)
 {
     if (k <= 16) return reduce_launch<8>(s, P, inv, n_beams, V, k, Y);
-    return k <= 32 ? reduce_launch<16>(s, P, inv, n_beams, V, k, Y) : reduce_launch<32>(s, P, inv, n_beams, V, k, Y);
+    if (k <= 32) return reduce_launch<16>(s, P, inv, n_beams, V, k, Y);
+    return launch_kernel(k_spmm_reduce_wide, (int)std::min<int64_t>((V * 32 + 255) / 256, kReduceBlocks), 256, 0, s, P, inv,
+                         n_beams, V, k, Y);
 }
 
 // inv[b][v] = position of voxel v in beam b's list (-1 if absent).
