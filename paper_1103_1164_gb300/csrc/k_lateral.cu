@@ -146,11 +146,12 @@ __device__ __forceinline__ float axis_taps_inside(const PlanView& P, const RhoQu
     return s;
 }
 
-// Whether the axis' taps, which are monotone in s, lie in [0, n - 1) of one grid axis.
+// Whether the axis' taps, which are monotone in s, lie in [0, n - 1) of one grid axis
+// (of at most 2^23 voxels, past which axis_taps_inside's whole parts are not exact).
 __device__ __forceinline__ bool taps_inside(float d, float e, float r, float o, float inv, int n)
 {
     const float u0 = tap_at((0.f - 7.5f) * d, e, r, o, inv), u1 = tap_at((15.f - 7.5f) * d, e, r, o, inv);
-    return fminf(u0, u1) >= 0.f && fmaxf(u0, u1) < (float)(n - 1);
+    return n <= 1 << 23 && fminf(u0, u1) >= 0.f && fmaxf(u0, u1) < (float)(n - 1);
 }
 
 // Effective densities of the axis stencil: (mean of the axis averages, x, y).
