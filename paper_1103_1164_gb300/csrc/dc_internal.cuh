@@ -81,7 +81,6 @@ struct dc_plan {
     float4* d_flupack = nullptr;     // the fluences of one multi-vector pass, [B][vectors]
     size_t flupack_cap = 0;          // floats
     int32_t* d_bcount = nullptr;     // per-beam pair counts [n_beams][V]
-    int persist_ctas[4] = {0, 0, 0, 0};
     // bumped whenever a buffer or a launch parameter that a captured batch
     // graph holds changes (binning geometry, partial-dose buffer, lateral form)
     uint64_t layout_gen = 0;

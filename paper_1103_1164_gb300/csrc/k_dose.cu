@@ -34,12 +34,12 @@ constexpr float kLog2e = 1.4426950408889634f;
 // needs moving when only its head is written out
 constexpr int kRing = 16;
 constexpr int kRingLd = kRing + 1;
+// (the values are what a profiler's kernel filter matches)
+enum Mode { kDose = 0, kFill = 2, kGrad = 3 };
 // beamlet records of a row window staged per warp at a time: fewer in the
 // fill, whose CSR staging shares the CTA's shared memory, and with more than
 // 32 fluence vectors, whose staging does
-constexpr int row_max(int mode, int nf = 1) { return mode == 2 || nf > 32 ? 16 : 32; }
-
-enum Mode { kDose = 0, kFill = 2, kGrad = 3 };
+constexpr int row_max(int mode, int nf = 1) { return mode == kFill || nf > 32 ? 16 : 32; }
 
 // PREC 2, the tensor-core form of the multi-fluence dose (64 vectors): per
 // warp and chunk of 16 beamlets, Y[32 voxels][64] += D[32][16] F[16][64] as
@@ -2299,24 +2299,9 @@ cudaError_t launch_dose(const dc_plan* p, const float* fluence, int nf, int ldf,
 
 cudaError_t launch_count(const dc_plan* p, int32_t* counts)
 {
-    DoseArgs a = make_args(p);
     cudaError_t e = cudaMemsetAsync(p->d_bcount, 0, sizeof(int32_t) * (size_t)p->n_beams * p->V, p->stream);
-    if (e != cudaSuccess) return e;
-    {
-        auto kern = k_count_units<kCountVoxels>;
-        int per_sm = 0, sms = 0;
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kThreads, 0);
-        if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, p->device);
-        if (e == cudaSuccess) e = cudaMemsetAsync(p->d_work + 1, 0, sizeof(int32_t), p->stream);
-        if (e != cudaSuccess) return e;
-        kern<<<sms * (per_sm > 0 ? per_sm : 1), kThreads, 0, p->stream>>>(a);
-        count_launches(1);
-        e = cudaGetLastError();
-    }
-    if (e != cudaSuccess) return e;
-    k_rowsum<<<grid_for(p->V), 256, 0, p->stream>>>(p->d_bcount, p->n_beams, p->V, counts);
-    count_launches(1);
-    return cudaGetLastError();
+    if (e == cudaSuccess) e = launch_units(p, k_count_units<kCountVoxels>, 0, make_args(p));
+    return e == cudaSuccess ? launch_rowsum(p, counts) : e;
 }
 
 cudaError_t launch_rowsum(const dc_plan* p, int32_t* counts)
