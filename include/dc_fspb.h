@@ -320,7 +320,9 @@ dc_status dc_fspb_spmm_noalloc(dc_plan* plan, const float* F, int32_t k, float* 
 dc_status dc_fspb_set_surrogate(dc_plan* plan, const float* params, float rho_lo, float rho_hi);
 
 /* Selects the lateral form (DC_LATERAL_*; DC_LATERAL_MLP needs
- * dc_fspb_set_surrogate first) and recomputes the per-entry factors.
+ * dc_fspb_set_surrogate first) and recomputes the per-entry factors.  A plan's
+ * first DC_LATERAL_AXIS allocates 16 bytes of device memory per voxel; without
+ * them the same factors take longer.
  * Asynchronous on the plan's stream.  Errors: DC_EINVAL, DC_ECUDA. */
 dc_status dc_fspb_set_lateral_mode(dc_plan* plan, int32_t mode);
 

@@ -122,16 +122,16 @@ struct DoseArgs {
     int32_t* cols;
     void* vals;
     int value_dtype;
+    int grad_shift;         // backward pass: log2 of the work items per unit
     const int32_t* items;   // beam voxel lists (k_bin.cu)
     const int64_t* base;    // [n_beams + 1]
     int32_t* work;          // [0] work units, [1] counter
     // backward pass with respect to the commissioning tables: voxel weights
-    // [V], the gradients [4][w_n], [4][f_n], [2] and log2 of the work items per unit
+    // [V] and the gradients [4][w_n], [4][f_n], [2]
     const float* wv;
     float* g_water;
     float* g_dens;
     float* g_corr;
-    int grad_shift;
 };
 
 }  // namespace dc

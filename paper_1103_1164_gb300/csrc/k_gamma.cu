@@ -16,7 +16,8 @@
 // kernel to finish folds the blocks' partials, and the statistics are taken as
 // gamma is computed.  With five kernels, a wait for the maximum between them and
 // five device blocks allocated and freed per call, a comparison on 128 x 128 x 96
-// voxels took 297 us, of which 45 us were kernels; now 95 us, of which 36 are.
+// voxels took 297 us, of which 45 us were kernels; now 88 to 111, of which 36 are (on
+// a host whose launches take longer, 351 and 149).
 #include <math.h>
 #include <stdint.h>
 #include <string.h>
